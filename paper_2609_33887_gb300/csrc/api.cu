@@ -511,12 +511,7 @@ int run_step(const Call& c, const BandPlan& plan, const Layout& lay, uint8_t* ws
   int* pa = reinterpret_cast<int*>(ws + lay.pa);
   const int P = static_cast<int>(c.P), d = static_cast<int>(c.d);
 
-  if (out_counts && !emit) {
-    if (cudaMemsetAsync(out_counts, 0, sizeof(int32_t) * size_t(c.n_seq) * c.T, st) != cudaSuccess)
-      return BD_ERR_CUDA;
-  }
-
-  // a0: compaction of the masked positions of active blocks (+ packing of their rows)
+  // a0: compaction of the masked positions of active blocks (+ packing of their rows; the counts cleared)
   // W8A8: the packed rows are quantised to E4M3 with one scale per row; a
   // head decoded inside the LM head: f16 rows scaled by a power of two per row
   const int row_format = c.fp8_act ? bd::ROWS_E4M3
@@ -525,10 +520,26 @@ int run_step(const Call& c, const BandPlan& plan, const Layout& lay, uint8_t* ws
                                    : bd::ROWS_BF16;
   float* tsc = row_format != bd::ROWS_BF16 ? reinterpret_cast<float*>(ws + lay.tsc) : nullptr;
   const int64_t ld_rows = (c.fp8_act || c.split) ? ld_fp8_rows(c) : c.ldc;
-  int rc = cuda_status(bd::launch_prep_rows(mask_state->pos_masked, mask_state->block_flags, P, c.L,
-                                            c.tc ? hidden->data : nullptr, c.ldh, d, c.tc ? ws + lay.hc : nullptr,
-                                            ld_rows, idx, rowpos, n_rows, sm_count, st, plan, tsc, row_format,
-                                            status));
+  bd::PrepArgs prep;
+  prep.pos_masked = mask_state->pos_masked;
+  prep.block_flags = mask_state->block_flags;
+  prep.P = P;
+  prep.block_len = c.L;
+  prep.chunk = 0;
+  prep.hidden = c.tc ? static_cast<const __nv_bfloat16*>(hidden->data) : nullptr;
+  prep.ld = c.ldh;
+  prep.d = d;
+  prep.hc = c.tc ? ws + lay.hc : nullptr;
+  prep.ldc = ld_rows;
+  prep.idx = idx;
+  prep.rowpos = rowpos;
+  prep.n_rows = n_rows;
+  prep.tok_scale = tsc;
+  prep.counts = emit ? nullptr : out_counts;
+  prep.n_counts = prep.counts ? c.n_seq * c.T : 0;
+  prep.status = status;
+  prep.plan = plan;
+  int rc = cuda_status(bd::launch_prep_rows(prep, row_format, sm_count, st));
   if (rc != BD_OK) return rc;
 
   rc = launch_lmhead(c, plan, hidden, weight, ws + lay.hc, ld_rows, ws + lay.wq, idx, n_rows, nullptr,

@@ -60,7 +60,7 @@ constexpr float FUSED_SHIFT_LIMIT = 2048.f;
 // once), then the smaller makespan, then the smaller gv; over GM <= min(n_mt,
 // G) with GM m-tiles of rows within the in-flight budget below (they stay in
 // L2 while their parts run) and gv <= min(G, n_vt). N is only known on the
-// device: the compaction kernel evaluates the rule with one warp and stores
+// device: one CTA of the compaction kernel evaluates the rule and stores
 // the plan beside N in the workspace header (HDR_* below), which the LM-head
 // and merge kernels read.
 // -------------------------------------------------------------------------
@@ -224,56 +224,71 @@ __host__ __device__ __forceinline__ void plan_choose(const BandPlan& p, int n_ro
 }
 
 #ifdef __CUDACC__
-// The same choice by a whole warp, 32 candidates at a time (the kernel that
-// learns N calls it once and stores GM and gv in the workspace header).
-__device__ __forceinline__ void plan_choose_warp(const BandPlan& p, int n_rows, int* gm_out, int* gv_out) {
+// One word per warp of the CTA that evaluates the plan.
+struct PlanScratch {
+  uint64_t w[32];
+};
+
+// The smallest v over the CTA's threads.
+__device__ __forceinline__ uint64_t cta_min(uint64_t v, PlanScratch* sh) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t other = __shfl_xor_sync(0xffffffffu, v, o);
+    v = other < v ? other : v;
+  }
+  __syncthreads();  // the scratch's previous use is over
+  if ((threadIdx.x & 31) == 0) sh->w[threadIdx.x >> 5] = v;
+  __syncthreads();
+  for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) v = sh->w[i] < v ? sh->w[i] : v;
+  return v;
+}
+
+// The same choice by a whole CTA, a candidate per thread (the kernel that
+// learns N calls it once and stores GM and gv in the workspace header). The
+// LM head waits for it: with 256 threads instead of one warp the 912
+// candidates of a 77-row float32 window take a few microseconds of what was a
+// 29.7 us kernel.
+__device__ __forceinline__ void plan_choose_cta(const BandPlan& p, int n_rows, int* gm_out, int* gv_out,
+                                                PlanScratch* sh) {
   const int n_mt = plan_runner_mts(p, n_rows) > 0 ? plan_runner_mts(p, n_rows) : 1;
   int glo, ghi, vlo, vhi;
   plan_gm_range(p, plan_bm(p, n_rows), n_mt, &glo, &ghi);
   plan_gv_range(p, &vlo, &vhi);
   const int nv = vhi - vlo + 1;
   const int total = (ghi - glo + 1) * nv;
-  const int lane = static_cast<int>(threadIdx.x & 31);
-  // the first 32 * CACHED candidates' costs stay in registers for the second pass
+  const int t = static_cast<int>(threadIdx.x), nt = static_cast<int>(blockDim.x);
+  // the first CACHED candidates of a thread keep their costs in registers for the second pass
   constexpr int CACHED = 4;
   uint64_t cc[CACHED];
   uint64_t c_min = ~uint64_t(0);
 #pragma unroll
   for (int q = 0; q < CACHED; ++q) {
-    const int i = lane + 32 * q;
+    const int i = t + nt * q;
     cc[q] = i < total ? plan_cost(p, n_mt, glo + i / nv, vlo + i % nv) : ~uint64_t(0);
     c_min = cc[q] < c_min ? cc[q] : c_min;
   }
-  for (int i = lane + 32 * CACHED; i < total; i += 32) {
+  for (int i = t + nt * CACHED; i < total; i += nt) {
     const uint64_t c = plan_cost(p, n_mt, glo + i / nv, vlo + i % nv);
     c_min = c < c_min ? c : c_min;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t other = __shfl_xor_sync(0xffffffffu, c_min, o);
-    c_min = other < c_min ? other : c_min;
-  }
+  c_min = cta_min(c_min, sh);
   const uint64_t c_max = c_min + c_min / MAKESPAN_SLACK_DIV;
   uint64_t best = ~uint64_t(0);
 #pragma unroll
   for (int q = 0; q < CACHED; ++q) {
-    const int i = lane + 32 * q;
+    const int i = t + nt * q;
     if (i < total && cc[q] <= c_max) {
       const uint64_t k = plan_key(p, n_mt, glo + i / nv, vlo + i % nv, cc[q]);
       best = k < best ? k : best;
     }
   }
-  for (int i = lane + 32 * CACHED; i < total; i += 32) {
+  for (int i = t + nt * CACHED; i < total; i += nt) {
     const uint64_t c = plan_cost(p, n_mt, glo + i / nv, vlo + i % nv);
     if (c > c_max) continue;
     const uint64_t k = plan_key(p, n_mt, glo + i / nv, vlo + i % nv, c);
     best = k < best ? k : best;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t other = __shfl_xor_sync(0xffffffffu, best, o);
-    best = other < best ? other : best;
-  }
+  best = cta_min(best, sh);
   *gm_out = static_cast<int>(best & 1023u);
   *gv_out = static_cast<int>((best >> 10) & 1023u);
 }
@@ -353,14 +368,14 @@ __host__ __device__ __forceinline__ void plan_header(const BandPlan& p, int n_ro
 }
 
 #ifdef __CUDACC__
-// The same header by one warp (the kernel that learns N calls it once); lane
+// The same header by one CTA (the kernel that learns N calls it once); thread
 // 0 writes it.
-__device__ __forceinline__ void plan_write_header(const BandPlan& p, int n_rows, int* hdr) {
+__device__ __forceinline__ void plan_write_header(const BandPlan& p, int n_rows, int* hdr, PlanScratch* sh) {
   const int vsplit = plan_vsplit(p, n_rows);
   int gm = 1, gv = 1, gm2 = 0, gv2 = 0;
-  plan_choose_warp(plan_share(p, vsplit, 0), n_rows, &gm, &gv);
-  if (vsplit < p.n_vt) plan_choose_warp(plan_share(p, vsplit, 1), n_rows, &gm2, &gv2);
-  if ((threadIdx.x & 31) == 0) plan_fill_header(p, n_rows, vsplit, gm, gv, gm2, gv2, hdr);
+  plan_choose_cta(plan_share(p, vsplit, 0), n_rows, &gm, &gv, sh);
+  if (vsplit < p.n_vt) plan_choose_cta(plan_share(p, vsplit, 1), n_rows, &gm2, &gv2, sh);
+  if (threadIdx.x == 0) plan_fill_header(p, n_rows, vsplit, gm, gv, gm2, gv2, hdr);
 }
 #endif
 

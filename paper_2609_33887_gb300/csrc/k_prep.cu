@@ -12,28 +12,71 @@ namespace bd {
 // active blocks). Rows keep ascending position order, so the masked positions
 // of a block are consecutive rows.
 //
-// CTA c owns positions [c*chunk, (c+1)*chunk). It counts the live positions
-// before its chunk itself (no inter-CTA communication), scans its chunk, writes
-// idx / rowpos for it, copies the hidden rows of its live positions into hc
-// (bf16 tensor-core paths) and, if it holds the last position, writes N.
+// CTA 0 counts the live positions of the whole window, clears the per-sequence
+// counts and writes the workspace header (N and the LM head's plan for N) with
+// all its threads. CTA 1 + c owns positions [c * chunk, (c + 1) * chunk): it
+// counts the live positions before its chunk itself (no inter-CTA
+// communication), scans its chunk, writes idx / rowpos for it and packs the
+// hidden rows of its live positions into hc (tensor-core paths), one warp per
+// row with the whole row's loads in flight.
+//
+// Bound: latency on small windows, where the LM head waits for this kernel.
+// Chunks are therefore as small as eight positions (a row per warp) until the
+// grid has four CTAs per SM.
 // ---------------------------------------------------------------------------
 constexpr int PREP_THREADS = 256;
+constexpr int PREP_WARPS = PREP_THREADS / 32;
+constexpr int PREP_MAX_CHUNK = 2048;
 
 __device__ __forceinline__ int live_at(const uint8_t* __restrict__ pos_masked, const uint8_t* __restrict__ block_flags,
                                        int p, int block_len) {
   return (pos_masked[p] != 0 && (block_flags[p / block_len] & 1u)) ? 1 : 0;
 }
 
-__device__ __forceinline__ int block_sum(int v, int* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// This thread's share of the live positions in [0, n): 16 mask bytes per load
+// where the array starts on a 16-byte boundary.
+__device__ __forceinline__ int count_live(const uint8_t* __restrict__ pos_masked,
+                                          const uint8_t* __restrict__ block_flags, int n, int block_len) {
+  int cnt = 0;
+  int done = 0;
+  if ((reinterpret_cast<uintptr_t>(pos_masked) & 15u) == 0) {
+    const int nv = n / 16;
+    const uint4* m4 = reinterpret_cast<const uint4*>(pos_masked);
+    for (int v = threadIdx.x; v < nv; v += PREP_THREADS) {
+      const uint4 q = __ldg(m4 + v);
+      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+      int b = 16 * v / block_len;
+      int rem = 16 * v - b * block_len;  // position within block b
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (rem + 4 <= block_len) {  // the four positions lie in one block
+          if (block_flags[b] & 1u) cnt += __popc(__vcmpne4(w[j], 0u)) >> 3;
+          rem += 4;
+          if (rem == block_len) {
+            rem = 0;
+            ++b;
+          }
+        } else {
+          for (int i = 0; i < 4; ++i) {
+            if (((w[j] >> (8 * i)) & 0xFFu) != 0 && (block_flags[b] & 1u)) ++cnt;
+            if (++rem == block_len) {
+              rem = 0;
+              ++b;
+            }
+          }
+        }
+      }
+    }
+    done = nv * 16;
+  }
+  for (int p = done + threadIdx.x; p < n; p += PREP_THREADS) cnt += live_at(pos_masked, block_flags, p, block_len);
+  return cnt;
+}
+
+__device__ __forceinline__ int warp_sum(int v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  int t = 0;
-  for (int w = 0; w < PREP_THREADS / 32; ++w) t += red[w];
-  __syncthreads();
-  return t;
+  return v;
 }
 
 // Two float32 values -> two E4M3 codes (round to nearest even, saturating at
@@ -49,167 +92,178 @@ __device__ __forceinline__ float2 f16x2_bits_to_float2(uint32_t h2) {
   return __half22float2(*reinterpret_cast<const __half2*>(&h2));
 }
 
-template <int FMT>  // the packed row format (ROWS_*); one instantiation per format
-__global__ void __launch_bounds__(PREP_THREADS) prep_rows_kernel(
-    const uint8_t* __restrict__ pos_masked, const uint8_t* __restrict__ block_flags, int P, int block_len, int chunk,
-    const __nv_bfloat16* __restrict__ hidden, int64_t ld, int d, __nv_bfloat16* __restrict__ hc, int64_t ldc,
-    int* __restrict__ idx, int* __restrict__ rowpos, int* __restrict__ n_rows, float* __restrict__ tok_scale,
-    uint32_t* __restrict__ status, BandPlan plan) {
-  __shared__ int red[PREP_THREADS / 32];
-  __shared__ int warp_excl[PREP_THREADS / 32];
-  __shared__ int rows_s[2048];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  griddep_launch_dependents();  // every CTA of this grid is resident once all have got here
-  const int p0 = blockIdx.x * chunk;
-  const int p1 = min(P, p0 + chunk);
+__device__ __forceinline__ float2 bf16x2_bits_to_float2(uint32_t b2) {
+  return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&b2));
+}
 
-  // 1. live positions before this chunk
-  int before = 0;
-  for (int p = tid; p < p0; p += PREP_THREADS) before += live_at(pos_masked, block_flags, p, block_len);
-  const int prefix = block_sum(before, red);
+__device__ __forceinline__ float amax8(const uint4& q) {
+  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+  float m = 0.f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float2 f = bf16x2_bits_to_float2(w[j]);
+    m = fmaxf(m, fmaxf(fabsf(f.x), fabsf(f.y)));
+  }
+  return m;
+}
 
-  // 2. exclusive scan of the chunk: thread t takes `per` consecutive positions
-  const int per = (chunk + PREP_THREADS - 1) / PREP_THREADS;
-  const int q0 = p0 + tid * per;
-  int cnt = 0;
-  for (int i = 0; i < per; ++i) {
-    const int p = q0 + i;
-    if (p < p1) cnt += live_at(pos_masked, block_flags, p, block_len);
-  }
-  int incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  if (lane == 31) warp_excl[warp] = incl;
-  __syncthreads();
-  if (tid == 0) {
-    int run = 0;
-    for (int w = 0; w < PREP_THREADS / 32; ++w) {
-      const int t = warp_excl[w];
-      warp_excl[w] = run;
-      run += t;
-    }
-    red[0] = run;  // live positions of the chunk
-  }
-  __syncthreads();
-  const int local_total = red[0];
-  int r = prefix + warp_excl[warp] + incl - cnt;
-  for (int i = 0; i < per; ++i) {
-    const int p = q0 + i;
-    if (p < p1) {
-      if (live_at(pos_masked, block_flags, p, block_len)) {
-        if (index_ok(r, P, status)) idx[r] = p;
-        rowpos[p] = r;
-        if (r - prefix < 2048) rows_s[r - prefix] = p;
-        ++r;
-      } else {
-        rowpos[p] = -1;
-      }
-    }
-  }
-  // The CTA holding the last position knows N: its warp 0 writes N and the
-  // plan for it into the header the later kernels read, while the CTA's other
-  // warps pack its rows (the plan's evaluation stays off the packing's path).
-  const bool header_warp = p1 == P && warp == 0;
-  if (hidden == nullptr) {
-    if (header_warp) plan_write_header(plan, prefix + local_total, n_rows);
-    return;
-  }
-  __syncthreads();
-  if (header_warp) {
-    plan_write_header(plan, prefix + local_total, n_rows);
-    return;
-  }
-  // the packing warps: all of them, or all but warp 0 in the header's CTA
-  const int w0 = p1 == P ? 1 : 0;
-  const int n_pack = PREP_THREADS / 32 - w0;
+// One packed row in the making: `up` multiplies the elements, and eight
+// (store8) or one (store1) of them are written in the format's codes.
+template <int FMT>
+struct RowOut {
+  uint8_t* hi;  // the packed row (ROWS_E4M3X2: its hi terms)
+  uint8_t* lo;  // ROWS_E4M3X2: its lo terms
+  float up;
 
-  const int nvec = d / 8;
-  if constexpr (FMT == ROWS_F16_POW2) {
-    // 3''. f16 rows for an LM head whose operands are f16: row r holds
-    // h * 2^s with s = 15 - e for max |h| in [2^(e-1), 2^e) (so the largest
-    // magnitude lands in [2^14, 2^15) and every bf16 value at or above 2^-14
-    // after scaling is exact in f16), s at most 126 so 2^-s stays a normal
-    // float; tok_scale = 2^-s, 0 for an all-zero row.
-    for (int i = warp - w0; i < local_total; i += n_pack) {
-      if (!index_ok(prefix + i, P, status)) continue;
-      const int p = i < 2048 ? rows_s[i] : idx[prefix + i];
-      const __nv_bfloat16* src = hidden + static_cast<int64_t>(p) * ld;
-      const uint4* s4 = reinterpret_cast<const uint4*>(src);
-      float amax = 0.f;
-#pragma unroll 4
-      for (int v = lane; v < nvec; v += 32) {
-        const uint4 q = __ldg(s4 + v);
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
-          amax = fmaxf(amax, fmaxf(fabsf(f.x), fabsf(f.y)));
-        }
-      }
-      for (int e = nvec * 8 + lane; e < d; e += 32) amax = fmaxf(amax, fabsf(__bfloat162float(src[e])));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-      // biased exponent E of amax: amax in [2^(E-127), 2^(E-126)) for E > 0,
-      // so s = 15 - (E - 126); E = 0 (zero or below 2^-126) takes the cap
-      const int E = static_cast<int>(__float_as_uint(amax) >> 23);
-      const int sh = amax > 0.f ? min(141 - E, 126) : 0;
-      const float up = __uint_as_float(static_cast<uint32_t>(sh + 127) << 23);  // 2^s, exact
-      __half* dst = reinterpret_cast<__half*>(hc) + static_cast<int64_t>(prefix + i) * ldc;
-      uint4* d4 = reinterpret_cast<uint4*>(dst);
-#pragma unroll 4
-      for (int v = lane; v < nvec; v += 32) {
-        const uint4 q = __ldg(s4 + v);
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-        uint32_t o[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
-          const __half2 h2 = __floats2half2_rn(f.x * up, f.y * up);
-          o[j] = *reinterpret_cast<const uint32_t*>(&h2);
-        }
-        d4[v] = make_uint4(o[0], o[1], o[2], o[3]);
-      }
-      for (int e = nvec * 8 + lane; e < d; e += 32) dst[e] = __float2half_rn(__bfloat162float(src[e]) * up);
-      if (lane == 0) tok_scale[prefix + i] = amax > 0.f ? __uint_as_float(static_cast<uint32_t>(127 - sh) << 23) : 0.f;
-    }
-    return;
-  }
-  if constexpr (FMT == ROWS_E4M3X2) {
-    // 3'''. bf16 rows as two E4M3 terms for an E4M3 head on the 8-bit tensor
-    // path (W8A16): row r is scaled by 2^s so that its largest magnitude lands
-    // in [128, 256) (s = 134 - E for the biased exponent E of max |h|, between
-    // -126 and 126 so 2^s and 2^-s stay normal floats; exact), then
-    // y = h * 2^s becomes hi = e4m3(y) and lo = e4m3(y - hi), both rounded to
-    // nearest even. y has at most 8 significant bits and y - hi (exact in
-    // float32) at most 4 more, so hi + lo == y exactly whenever |y| >= 2^-2,
-    // i.e. for every element of at least 2^-10 times the row's largest; a
-    // smaller element is off by at most 2^-10 (half the smallest E4M3 step),
-    // 2^-17 of the row's largest. hi rows at hc, lo rows at hc + P * ldc (ldc
-    // in bytes); tok_scale = 2^-s (0 for an all-zero row).
-    uint8_t* hq = reinterpret_cast<uint8_t*>(hc);
-    uint8_t* lq = hq + static_cast<int64_t>(P) * ldc;
-    // rows of up to 32 * RC vectors (5120 bf16) are read once, into
-    // registers: every lane's loads of the row are in flight together
-    constexpr int RC = 20;
-    const bool cached = nvec <= 32 * RC;
-    auto amax_of = [](const uint4& q) {
-      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-      float m = 0.f;
+  __device__ __forceinline__ void store8(const uint4& q, int v) const {
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    if constexpr (FMT == ROWS_F16_POW2) {
+      uint32_t o[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
-        m = fmaxf(m, fmaxf(fabsf(f.x), fabsf(f.y)));
+        const float2 f = bf16x2_bits_to_float2(w[j]);
+        const __half2 h2 = __floats2half2_rn(f.x * up, f.y * up);
+        o[j] = *reinterpret_cast<const uint32_t*>(&h2);
       }
-      return m;
-    };
-    for (int i = warp - w0; i < local_total; i += n_pack) {
-      if (!index_ok(prefix + i, P, status)) continue;
-      const int p = i < 2048 ? rows_s[i] : idx[prefix + i];
-      const __nv_bfloat16* src = hidden + static_cast<int64_t>(p) * ld;
-      const uint4* s4 = reinterpret_cast<const uint4*>(src);
+      reinterpret_cast<uint4*>(hi)[v] = make_uint4(o[0], o[1], o[2], o[3]);
+    } else {
+      uint32_t oh[2] = {0u, 0u}, ol[2] = {0u, 0u};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 f = bf16x2_bits_to_float2(w[j]);
+        const float y0 = __fmul_rn(f.x, up), y1 = __fmul_rn(f.y, up);
+        const uint32_t h2 = f32x2_to_e4m3x2(y0, y1);
+        oh[j >> 1] |= h2 << (16 * (j & 1));
+        if constexpr (FMT == ROWS_E4M3X2) {
+          const float2 back = f16x2_bits_to_float2(e4m3x2_to_f16x2(h2));
+          ol[j >> 1] |= f32x2_to_e4m3x2(y0 - back.x, y1 - back.y) << (16 * (j & 1));
+        }
+      }
+      reinterpret_cast<uint2*>(hi)[v] = make_uint2(oh[0], oh[1]);
+      if constexpr (FMT == ROWS_E4M3X2) reinterpret_cast<uint2*>(lo)[v] = make_uint2(ol[0], ol[1]);
+    }
+  }
+
+  __device__ __forceinline__ void store1(float x, int e) const {
+    if constexpr (FMT == ROWS_F16_POW2) {
+      reinterpret_cast<__half*>(hi)[e] = __float2half_rn(x * up);
+    } else {
+      const float y = __fmul_rn(x, up);
+      const uint32_t h2 = f32x2_to_e4m3x2(y, 0.f);
+      hi[e] = static_cast<uint8_t>(h2 & 0xFFu);
+      if constexpr (FMT == ROWS_E4M3X2) {
+        const float back = f16x2_bits_to_float2(e4m3x2_to_f16x2(h2)).x;
+        lo[e] = static_cast<uint8_t>(f32x2_to_e4m3x2(y - back, 0.f) & 0xFFu);
+      }
+    }
+  }
+};
+
+// The factor a row of largest magnitude amax is multiplied by before it is
+// encoded, and the token scale that undoes it on the logits (0 for an all-zero row).
+//
+// ROWS_F16_POW2: 2^s with s = 15 - e for amax in [2^(e-1), 2^e), so the largest
+// magnitude lands in [2^14, 2^15) and every bf16 value at or above 2^-14 after
+// scaling is exact in f16; s at most 126 so 2^-s stays a normal float.
+//
+// ROWS_E4M3X2 (W8A16 on the 8-bit tensor path): 2^s with s = 134 - E for the
+// biased exponent E of amax (the largest magnitude lands in [128, 256)),
+// between -126 and 126 so 2^s and 2^-s stay normal floats. y = h * 2^s (exact)
+// becomes hi = e4m3(y) and lo = e4m3(y - hi), both rounded to nearest even. y
+// has at most 8 significant bits and y - hi (exact in float32) at most 4 more,
+// so hi + lo == y exactly whenever |y| >= 2^-2, i.e. for every element of at
+// least 2^-10 of the row's largest; a smaller element is off by at most 2^-10
+// (half the smallest E4M3 step), 2^-17 of the row's largest.
+//
+// ROWS_E4M3 (W8A8): 448 / amax, code = e4m3(h * inv), scale = amax / 448; each
+// float32 step is one correctly rounded operation.
+template <int FMT>
+__device__ __forceinline__ void row_factors(float amax, float* up, float* scale) {
+  if constexpr (FMT == ROWS_E4M3) {
+    *up = amax > 0.f ? __fdiv_rn(448.f, amax) : 0.f;
+    *scale = amax > 0.f ? __fdiv_rn(amax, 448.f) : 0.f;
+  } else {
+    const int E = static_cast<int>(__float_as_uint(amax) >> 23);
+    // amax in [2^(E-127), 2^(E-126)) for E > 0; E = 0 (zero or below 2^-126) takes the cap
+    const int sh = !(amax > 0.f) ? 0 : FMT == ROWS_F16_POW2 ? min(141 - E, 126) : max(min(134 - E, 126), -126);
+    *up = __uint_as_float(static_cast<uint32_t>(sh + 127) << 23);  // 2^s, exact
+    *scale = amax > 0.f ? __uint_as_float(static_cast<uint32_t>(127 - sh) << 23) : 0.f;
+  }
+}
+
+template <int FMT>  // the packed row format (ROWS_*); one instantiation per format
+__global__ void __launch_bounds__(PREP_THREADS) prep_rows_kernel(PrepArgs a) {
+  __shared__ int red[2][PREP_WARPS];
+  __shared__ int rows_s[PREP_MAX_CHUNK];
+  __shared__ PlanScratch plan_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  griddep_launch_dependents();  // every CTA of this grid is resident once all have got here
+  griddep_wait();               // the caller's window, and the previous step's use of the workspace
+
+  if (blockIdx.x == 0) {
+    // the header's CTA
+    const int cnt = warp_sum(count_live(a.pos_masked, a.block_flags, a.P, a.block_len));
+    if (lane == 0) red[0][warp] = cnt;
+    for (int i = tid; i < a.n_counts; i += PREP_THREADS) a.counts[i] = 0;
+    __syncthreads();
+    int n = 0;
+#pragma unroll
+    for (int w = 0; w < PREP_WARPS; ++w) n += red[0][w];
+    plan_write_header(a.plan, n, a.n_rows, &plan_s);
+    return;
+  }
+
+  const int p0 = (static_cast<int>(blockIdx.x) - 1) * a.chunk;
+  const int p1 = min(a.P, p0 + a.chunk);
+  // 1. live positions before this chunk, and the scan of the chunk, 256 positions at a time
+  const int before = warp_sum(count_live(a.pos_masked, a.block_flags, p0, a.block_len));
+  if (lane == 0) red[1][warp] = before;
+  int prefix = 0, local_total = 0;
+  for (int s0 = p0; s0 < p1; s0 += PREP_THREADS) {
+    const int p = s0 + tid;
+    const bool mine = p < p1 && live_at(a.pos_masked, a.block_flags, p, a.block_len);
+    const uint32_t bal = __ballot_sync(0xffffffffu, mine);
+    if (lane == 0) red[0][warp] = __popc(bal);
+    __syncthreads();
+    if (s0 == p0) {
+#pragma unroll
+      for (int w = 0; w < PREP_WARPS; ++w) prefix += red[1][w];
+    }
+    int excl = local_total;
+#pragma unroll
+    for (int w = 0; w < PREP_WARPS; ++w) {
+      const int c = red[0][w];
+      if (w < warp) excl += c;
+      local_total += c;
+    }
+    if (p < p1) {
+      const int i = excl + __popc(bal & ((1u << lane) - 1u));
+      if (mine) {
+        if (index_ok(prefix + i, a.P, a.status)) a.idx[prefix + i] = p;
+        rows_s[i] = p;
+      }
+      a.rowpos[p] = mine ? prefix + i : -1;
+    }
+    __syncthreads();
+  }
+  if (a.hidden == nullptr) return;
+
+  // 2. pack the chunk's live rows
+  const int d = a.d, nvec = d / 8;
+  for (int i = warp; i < local_total; i += PREP_WARPS) {
+    if (!index_ok(prefix + i, a.P, a.status)) continue;
+    const __nv_bfloat16* src = a.hidden + static_cast<int64_t>(rows_s[i]) * a.ld;
+    const uint4* s4 = reinterpret_cast<const uint4*>(src);
+    if constexpr (FMT == ROWS_BF16) {
+      __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(a.hc) + static_cast<int64_t>(prefix + i) * a.ldc;
+      uint4* d4 = reinterpret_cast<uint4*>(dst);
+#pragma unroll 8
+      for (int v = lane; v < nvec; v += 32) d4[v] = __ldg(s4 + v);
+      for (int e = nvec * 8 + lane; e < d; e += 32) dst[e] = src[e];
+    } else {
+      // rows of up to 32 * RC vectors (5120 bf16) are read once, into registers
+      constexpr int RC = 20;
+      const bool cached = nvec <= 32 * RC;
       uint4 qc[RC];
       float amax = 0.f;
       if (cached) {
@@ -219,149 +273,74 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_rows_kernel(
           qc[k] = v < nvec ? __ldg(s4 + v) : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
-        for (int k = 0; k < RC; ++k) amax = fmaxf(amax, amax_of(qc[k]));
+        for (int k = 0; k < RC; ++k) amax = fmaxf(amax, amax8(qc[k]));
       } else {
 #pragma unroll 4
-        for (int v = lane; v < nvec; v += 32) amax = fmaxf(amax, amax_of(__ldg(s4 + v)));
+        for (int v = lane; v < nvec; v += 32) amax = fmaxf(amax, amax8(__ldg(s4 + v)));
       }
       for (int e = nvec * 8 + lane; e < d; e += 32) amax = fmaxf(amax, fabsf(__bfloat162float(src[e])));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-      const int E = static_cast<int>(__float_as_uint(amax) >> 23);
-      const int sh = amax > 0.f ? max(min(134 - E, 126), -126) : 0;
-      const float up = __uint_as_float(static_cast<uint32_t>(sh + 127) << 23);  // 2^s, exact
-      uint8_t* dh = hq + static_cast<int64_t>(prefix + i) * ldc;
-      uint8_t* dl = lq + static_cast<int64_t>(prefix + i) * ldc;
-      // vector v of the row: eight elements as eight hi and eight lo codes
-      auto convert_store = [&](const uint4& q, int v) {
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-        uint32_t oh[2], ol[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          uint32_t h4 = 0, l4 = 0;
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[2 * j + u]));
-            const float y0 = f.x * up, y1 = f.y * up;
-            const uint32_t h2 = f32x2_to_e4m3x2(y0, y1);
-            const float2 back = f16x2_bits_to_float2(e4m3x2_to_f16x2(h2));
-            const uint32_t l2 = f32x2_to_e4m3x2(y0 - back.x, y1 - back.y);
-            h4 |= h2 << (16 * u);
-            l4 |= l2 << (16 * u);
-          }
-          oh[j] = h4;
-          ol[j] = l4;
-        }
-        *reinterpret_cast<uint2*>(dh + 8 * v) = make_uint2(oh[0], oh[1]);
-        *reinterpret_cast<uint2*>(dl + 8 * v) = make_uint2(ol[0], ol[1]);
-      };
+      // ldc counts bytes for the 8-bit formats, f16 elements for ROWS_F16_POW2
+      const int64_t row_bytes = FMT == ROWS_F16_POW2 ? 2 * a.ldc : a.ldc;
+      RowOut<FMT> out;
+      float scale;
+      row_factors<FMT>(amax, &out.up, &scale);
+      out.hi = static_cast<uint8_t*>(a.hc) + static_cast<int64_t>(prefix + i) * row_bytes;
+      out.lo = out.hi + static_cast<int64_t>(a.P) * row_bytes;
       if (cached) {
 #pragma unroll
         for (int k = 0; k < RC; ++k) {
           const int v = lane + 32 * k;
-          if (v < nvec) convert_store(qc[k], v);
+          if (v < nvec) out.store8(qc[k], v);
         }
       } else {
 #pragma unroll 4
-        for (int v = lane; v < nvec; v += 32) convert_store(__ldg(s4 + v), v);
+        for (int v = lane; v < nvec; v += 32) out.store8(__ldg(s4 + v), v);
       }
-      for (int e = nvec * 8 + lane; e < d; e += 32) {
-        const float y = __bfloat162float(src[e]) * up;
-        const uint32_t h2 = f32x2_to_e4m3x2(y, 0.f);
-        const float back = f16x2_bits_to_float2(e4m3x2_to_f16x2(h2)).x;
-        dh[e] = static_cast<uint8_t>(h2 & 0xFFu);
-        dl[e] = static_cast<uint8_t>(f32x2_to_e4m3x2(y - back, 0.f) & 0xFFu);
-      }
-      if (lane == 0) tok_scale[prefix + i] = amax > 0.f ? __uint_as_float(static_cast<uint32_t>(127 - sh) << 23) : 0.f;
+      for (int e = nvec * 8 + lane; e < d; e += 32) out.store1(__bfloat162float(src[e]), e);
+      if (lane == 0) a.tok_scale[prefix + i] = scale;
     }
-    return;
-  }
-  if constexpr (FMT == ROWS_E4M3) {
-    // 3'. W8A8: quantise the chunk's live rows to E4M3 with one scale per row,
-    // one warp per row: a = max |h|, inv = 448 / a, code = e4m3(h * inv) (round
-    // to nearest even, saturating), scale = a / 448; an all-zero row gets codes
-    // 0 and scale 0. Each float32 step is one correctly rounded operation.
-    uint8_t* hq = reinterpret_cast<uint8_t*>(hc);  // ldc counts bytes here
-    for (int i = warp - w0; i < local_total; i += n_pack) {
-      if (!index_ok(prefix + i, P, status)) continue;
-      const int p = i < 2048 ? rows_s[i] : idx[prefix + i];
-      const __nv_bfloat16* src = hidden + static_cast<int64_t>(p) * ld;
-      const uint4* s4 = reinterpret_cast<const uint4*>(src);
-      float amax = 0.f;
-#pragma unroll 4
-      for (int v = lane; v < nvec; v += 32) {
-        const uint4 q = __ldg(s4 + v);
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
-          amax = fmaxf(amax, fmaxf(fabsf(f.x), fabsf(f.y)));
-        }
-      }
-      for (int e = nvec * 8 + lane; e < d; e += 32) amax = fmaxf(amax, fabsf(__bfloat162float(src[e])));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-      const float inv = amax > 0.f ? __fdiv_rn(448.f, amax) : 0.f;
-      uint8_t* dst = hq + static_cast<int64_t>(prefix + i) * ldc;
-#pragma unroll 4
-      for (int v = lane; v < nvec; v += 32) {
-        const uint4 q = __ldg(s4 + v);
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-        uint32_t out[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[2 * j]));
-          const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[2 * j + 1]));
-          out[j] = f32x2_to_e4m3x2(__fmul_rn(f0.x, inv), __fmul_rn(f0.y, inv)) |
-                   (f32x2_to_e4m3x2(__fmul_rn(f1.x, inv), __fmul_rn(f1.y, inv)) << 16);
-        }
-        *reinterpret_cast<uint2*>(dst + 8 * v) = make_uint2(out[0], out[1]);
-      }
-      for (int e = nvec * 8 + lane; e < d; e += 32)
-        dst[e] = static_cast<uint8_t>(f32x2_to_e4m3x2(__fmul_rn(__bfloat162float(src[e]), inv), 0.f) & 0xFFu);
-      if (lane == 0) tok_scale[prefix + i] = amax > 0.f ? __fdiv_rn(amax, 448.f) : 0.f;
-    }
-    return;
-  }
-
-  // 3. copy the chunk's live rows, one warp per row, 16-byte vectors
-  for (int i = warp - w0; i < local_total; i += n_pack) {
-    if (!index_ok(prefix + i, P, status)) continue;
-    const int p = i < 2048 ? rows_s[i] : idx[prefix + i];
-    const __nv_bfloat16* src = hidden + static_cast<int64_t>(p) * ld;
-    __nv_bfloat16* dst = hc + static_cast<int64_t>(prefix + i) * ldc;
-    const uint4* s4 = reinterpret_cast<const uint4*>(src);
-    uint4* d4 = reinterpret_cast<uint4*>(dst);
-#pragma unroll 4
-    for (int v = lane; v < nvec; v += 32) d4[v] = __ldg(s4 + v);
-    for (int e = nvec * 8 + lane; e < d; e += 32) dst[e] = src[e];
   }
 }
 
+// Positions per packing CTA: four CTAs per SM, at least a row per warp.
 int prep_chunk(int P, int sm_count) {
-  int chunk = (P + 2 * sm_count - 1) / (2 * sm_count);
-  chunk = (chunk + 31) / 32 * 32;
-  if (chunk < 32) chunk = 32;
-  if (chunk > 2048) chunk = 2048;
-  return chunk;
+  int chunk = (P + 4 * sm_count - 1) / (4 * sm_count);
+  chunk = (chunk + PREP_WARPS - 1) / PREP_WARPS * PREP_WARPS;
+  return chunk > PREP_MAX_CHUNK ? PREP_MAX_CHUNK : chunk;
 }
 
-cudaError_t launch_prep_rows(const uint8_t* pos_masked, const uint8_t* block_flags, int P, int block_len,
-                             const void* hidden, int64_t ld, int d, void* hc, int64_t ldc, int* idx, int* rowpos,
-                             int* n_rows, int sm_count, cudaStream_t st, const BandPlan& plan, float* tok_scale,
-                             int row_format, uint32_t* status) {
-  if (row_format != ROWS_BF16 && (tok_scale == nullptr || hc == nullptr)) return cudaErrorInvalidValue;
-  const int chunk = prep_chunk(P, sm_count);
-  const int grid = (P + chunk - 1) / chunk;
+// Launched with programmatic stream serialisation behind the kernel before it
+// (every CTA waits for that kernel first), except into a stream capture, whose
+// first node may follow copies and other streams' work.
+template <typename... Params, typename... Args>
+static cudaError_t launch_behind(void (*kern)(Params...), int grid, cudaStream_t st, const Args&... args) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(st, &cs);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
+  cfg.blockDim = dim3(PREP_THREADS, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cs == cudaStreamCaptureStatusNone ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+cudaError_t launch_prep_rows(const PrepArgs& args, int row_format, int sm_count, cudaStream_t st) {
+  if (row_format != ROWS_BF16 && (args.tok_scale == nullptr || args.hc == nullptr)) return cudaErrorInvalidValue;
+  PrepArgs a = args;
+  a.chunk = prep_chunk(a.P, sm_count);
+  const int grid = 1 + (a.P + a.chunk - 1) / a.chunk;
   auto* kern = row_format == ROWS_F16_POW2 ? prep_rows_kernel<ROWS_F16_POW2>
                : row_format == ROWS_E4M3  ? prep_rows_kernel<ROWS_E4M3>
                : row_format == ROWS_E4M3X2 ? prep_rows_kernel<ROWS_E4M3X2>
                                            : prep_rows_kernel<ROWS_BF16>;
-  kern<<<grid, PREP_THREADS, 0, st>>>(pos_masked, block_flags, P, block_len, chunk,
-                                      static_cast<const __nv_bfloat16*>(hidden), ld, d,
-                                      static_cast<__nv_bfloat16*>(hc), ldc, idx, rowpos, n_rows, tok_scale, status,
-                                      plan);
-  return cudaGetLastError();
+  return launch_behind(kern, grid, st, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -369,27 +348,33 @@ cudaError_t launch_prep_rows(const uint8_t* pos_masked, const uint8_t* block_fla
 // r = q * (n_draft + 1) + i verifies draft token i of request q (i < n_draft);
 // the last row of a request verifies nothing.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) prep_verify_kernel(const int32_t* __restrict__ draft, int n_req, int n_draft,
-                                                          int* __restrict__ idx, int* __restrict__ draft_row,
-                                                          int* __restrict__ n_rows, BandPlan plan) {
+__global__ void __launch_bounds__(PREP_THREADS) prep_verify_kernel(const int32_t* __restrict__ draft, int n_req,
+                                                                   int n_draft, int* __restrict__ idx,
+                                                                   int* __restrict__ draft_row,
+                                                                   int* __restrict__ n_rows, BandPlan plan) {
+  __shared__ PlanScratch plan_s;
   griddep_launch_dependents();
+  griddep_wait();
   const int R = n_req * (n_draft + 1);
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
+  if (blockIdx.x == 0) {  // N and the plan for it
+    plan_write_header(plan, R, n_rows, &plan_s);
+    return;
+  }
+  const int step = (gridDim.x - 1) * PREP_THREADS;
+  for (int r = (blockIdx.x - 1) * PREP_THREADS + threadIdx.x; r < R; r += step) {
     const int q = r / (n_draft + 1), i = r % (n_draft + 1);
     idx[r] = r;
     draft_row[r] = i < n_draft ? draft[q * n_draft + i] : -1;
   }
-  if (blockIdx.x == 0 && threadIdx.x < 32) plan_write_header(plan, R, n_rows);  // N and the plan for it
 }
 
 cudaError_t launch_prep_verify(const int32_t* draft, int n_req, int n_draft, int* idx, int* draft_row, int* n_rows,
                                const BandPlan& plan, cudaStream_t st) {
   const int R = n_req * (n_draft + 1);
-  int grid = (R + 255) / 256;
+  int grid = (R + PREP_THREADS - 1) / PREP_THREADS;
   if (grid < 1) grid = 1;
   if (grid > 1024) grid = 1024;
-  prep_verify_kernel<<<grid, 256, 0, st>>>(draft, n_req, n_draft, idx, draft_row, n_rows, plan);
-  return cudaGetLastError();
+  return launch_behind(prep_verify_kernel, 1 + grid, st, draft, n_req, n_draft, idx, draft_row, n_rows, plan);
 }
 
 // ---------------------------------------------------------------------------

@@ -31,12 +31,26 @@ struct TauParams {
 // bytes, a multiple of 16), exact for every element of at least 2^-10 of the
 // row's largest; tok_scale[r] = 2^-s.
 enum : int { ROWS_BF16 = 0, ROWS_E4M3 = 1, ROWS_F16_POW2 = 2, ROWS_E4M3X2 = 3 };
-// n_rows: the workspace header (N and the LM head's plan for N, HDR_* words of
-// common.cuh), written by the CTA that holds the last position.
-cudaError_t launch_prep_rows(const uint8_t* pos_masked, const uint8_t* block_flags, int P, int block_len,
-                             const void* hidden, int64_t ld, int d, void* hc, int64_t ldc, int* idx, int* rowpos,
-                             int* n_rows, int sm_count, cudaStream_t st, const BandPlan& plan,
-                             float* tok_scale = nullptr, int row_format = ROWS_BF16, uint32_t* status = nullptr);
+struct PrepArgs {
+  const uint8_t* pos_masked;
+  const uint8_t* block_flags;
+  int P, block_len;
+  int chunk;  // positions per packing CTA (set by the launcher)
+  const __nv_bfloat16* hidden;
+  int64_t ld;
+  int d;
+  void* hc;
+  int64_t ldc;
+  int* idx;
+  int* rowpos;
+  int* n_rows;       // the workspace header (N and the LM head's plan for N, HDR_* words of common.cuh)
+  float* tok_scale;  // every format but ROWS_BF16
+  int32_t* counts;   // the step's per-sequence counts, cleared here (may be null)
+  int n_counts;
+  uint32_t* status;
+  BandPlan plan;
+};
+cudaError_t launch_prep_rows(const PrepArgs& a, int row_format, int sm_count, cudaStream_t st);
 
 // Decodes FP8 e4m3 weight codes to bf16 (exact), row by row: out[v] = code(w[v]).
 cudaError_t launch_dequant_e4m3(const uint8_t* w, int64_t ldw, int V, int d, void* out, int64_t ldo,
