@@ -272,8 +272,11 @@ int bd_plan_header(const bd_hidden* hidden, const bd_weight* weight, const bd_ma
  *                        head tile by multicast (default: clusters for windows of
  *                        at most 512 positions or more than 256 MiB of packed rows)
  *   BD_PAIR_SHARE=0|1    the two pairs of a cluster share head tiles (two token
- *                        groups, one v-tile at a time; default) or token rows (one
- *                        token group, two v-tiles at a time)
+ *                        groups, one v-tile at a time) or token rows (one token
+ *                        group, two v-tiles at a time); default: head tiles, or
+ *                        token rows where the window holds a single token group
+ *                        (at most 256 compacted rows; chosen on the device, unless
+ *                        BD_PAIR_MC is set)
  *   BD_PAIR_SPILL=0|1    with clusters of two pairs, the CTA pairs that still fit
  *                        on the SMs the clusters leave free (4 on a 152-SM GB300)
  *                        take the last v-tiles in a second, concurrent launch

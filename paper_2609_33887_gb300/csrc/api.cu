@@ -252,7 +252,8 @@ BandPlan make_plan(const Call& c, int sm_count, int pairs, int quads) {
       // the cluster's two pairs share head tiles (two token groups, one v-tile
       // at a time) or, with BD_PAIR_SHARE = 1, token rows (one token group,
       // two v-tiles at a time)
-      if (env_int("BD_PAIR_SHARE", 0, 0, 1) == 1) {
+      const int share = env_int("BD_PAIR_SHARE", -1, 0, 1);
+      if (share == 1) {
         p.mc = 1;
         p.vc = 2;
       }
@@ -266,6 +267,9 @@ BandPlan make_plan(const Call& c, int sm_count, int pairs, int quads) {
         p.G2 = spare;
         p.spill_pct = env_int("BD_SPILL_PCT", 100, 50, 400);
       }
+      // small windows may turn out to hold a single token group: the choice is
+      // then made on the device (plan_resolve), unless a layout is forced
+      if (share < 0 && env_int("BD_PAIR_MC", -1, 1, 2) < 0 && p.G2 == 0) p.adapt = 1;
     }
   } else if (c.tc) {
     p.BM = bd::TC_BM;
@@ -315,6 +319,18 @@ Layout make_layout(const Call& c, const BandPlan& p) {
   l.tsc = take(4 * P, 256);                                             // W8A8: per-row token scales
   l.wq = decoded_head(c) ? take(2 * static_cast<size_t>(c.ldq) * static_cast<size_t>(c.V), 1024) : 0;
   l.total = (off + 255) / 256 * 256;
+  return l;
+}
+
+// The plan and layout for a workspace of `bytes`: the device's choice between
+// the cluster layouts needs up to twice the partial slots, and is left out
+// where they do not fit.
+Layout fit_layout(const Call& c, BandPlan* p, size_t bytes) {
+  Layout l = make_layout(c, *p);
+  if (l.total > bytes && p->adapt) {
+    p->adapt = 0;
+    l = make_layout(c, *p);
+  }
   return l;
 }
 
@@ -682,8 +698,8 @@ int bd_commit_step_ex(const bd_hidden* hidden, const bd_weight* weight, const bd
   DevCtx* ctx = nullptr;
   rc = device_ctx(&ctx);
   if (rc != BD_OK) return rc;
-  const BandPlan plan = make_plan(c, ctx->sm_count, ctx->pairs, ctx->quads);
-  const Layout lay = make_layout(c, plan);
+  BandPlan plan = make_plan(c, ctx->sm_count, ctx->pairs, ctx->quads);
+  const Layout lay = fit_layout(c, &plan, exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX);
 
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {
@@ -737,8 +753,8 @@ int bd_lmhead_partials(const bd_hidden* hidden, const bd_weight* shard, int64_t 
   DevCtx* ctx = nullptr;
   rc = device_ctx(&ctx);
   if (rc != BD_OK) return rc;
-  const BandPlan plan = make_plan(c, ctx->sm_count, ctx->pairs, ctx->quads);
-  const Layout lay = make_layout(c, plan);
+  BandPlan plan = make_plan(c, ctx->sm_count, ctx->pairs, ctx->quads);
+  const Layout lay = fit_layout(c, &plan, exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX);
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {
     if (exec->workspace_bytes < lay.total) return BD_ERR_WORKSPACE;
@@ -949,8 +965,8 @@ extern "C" int bd_commit_step_static(const bd_hidden* hidden, const bd_weight* w
   StaticCtx* sctx = nullptr;
   rc = static_ctx(&sctx);
   if (rc != BD_OK) return rc;
-  const BandPlan plan = make_plan(c, sctx->sm_count, sctx->pairs, sctx->quads);
-  const Layout lay = make_layout(c, plan);
+  BandPlan plan = make_plan(c, sctx->sm_count, sctx->pairs, sctx->quads);
+  const Layout lay = fit_layout(c, &plan, BD_STATIC_SCRATCH_BYTES);
   if (lay.total > BD_STATIC_SCRATCH_BYTES) return BD_ERR_WORKSPACE;
 
   uint8_t* ws = sctx->scratch;
@@ -1140,8 +1156,12 @@ int bd_verify_step(const bd_hidden* hidden, const bd_weight* weight, const bd_dr
   DevCtx* ctx = nullptr;
   rc = device_ctx(&ctx);
   if (rc != BD_OK) return rc;
-  const BandPlan plan = make_plan(vc.c, ctx->sm_count, ctx->pairs, ctx->quads);
-  const VerifyLayout lay = make_verify_layout(vc.c, plan);
+  BandPlan plan = make_plan(vc.c, ctx->sm_count, ctx->pairs, ctx->quads);
+  VerifyLayout lay = make_verify_layout(vc.c, plan);
+  if (exec && exec->workspace && exec->workspace_bytes < lay.total && plan.adapt) {
+    plan.adapt = 0;  // as fit_layout
+    lay = make_verify_layout(vc.c, plan);
+  }
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {
     if (exec->workspace_bytes < lay.total) return BD_ERR_WORKSPACE;

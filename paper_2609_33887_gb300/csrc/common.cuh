@@ -75,6 +75,7 @@ struct BandPlan {
   int row_bytes;  // bytes of one packed token row as the kernel reads it
   int mc;         // m-tiles a runner holds at once (1, or 2 for 4-CTA clusters sharing head tiles)
   int vc;         // v-tiles a runner takes at once (1, or 2 for 4-CTA clusters sharing token rows)
+  int adapt;      // 1: clusters with mc = 2 take vc = 2 instead while the rows form a single token group
   int gv_fixed;   // vocabulary parts when > 0 (clamped to 1..min(G, n_vt)), else chosen
   int rr;         // 1: units taken round-robin (runner c: units c, c + G, ...) instead of packed rounds
   int G2;         // spill runners: single CTA pairs on the SMs the clusters leave free (0: none)
@@ -109,6 +110,23 @@ __host__ __device__ __forceinline__ int plan_bm(const BandPlan& p, int n_rows) {
 
 __host__ __device__ __forceinline__ int plan_mc(const BandPlan& p) { return p.mc > 1 ? p.mc : 1; }
 __host__ __device__ __forceinline__ int plan_vc(const BandPlan& p) { return p.vc > 1 ? p.vc : 1; }
+
+// The plan once N is known. With two pairs per cluster and a single token
+// group, sharing head tiles would leave the second pair multiplying zero rows:
+// the pairs share the group's rows and take two v-tiles instead. 8 x 2 x 32
+// windows with every other position resolved (N = 256, d = 2048, V = 151936),
+// LM head before and after: bf16 170 -> 115 us, E4M3 162 -> 101 us, W8A8
+// 104 -> 68 us; N = 128: 117 -> 100, 88 -> 59, 74 -> 57 us. With two groups
+// (N = 257..512) sharing head tiles stays faster: 146 against 152 us a step at
+// N = 294 in bf16, 135 against 144 us with an E4M3 head.
+__host__ __device__ __forceinline__ BandPlan plan_resolve(const BandPlan& p, int n_rows) {
+  BandPlan q = p;
+  if (p.adapt && n_rows <= 256) {
+    q.mc = 1;
+    q.vc = 2;
+  }
+  return q;
+}
 
 // Runner m-tiles (of plan_mc m-tiles each) for N rows; 0 without rows.
 __host__ __device__ __forceinline__ int plan_runner_mts(const BandPlan& p, int n_rows) {
@@ -359,7 +377,8 @@ __host__ __device__ __forceinline__ void plan_fill_header(const BandPlan& p, int
 }
 
 // The workspace header for N rows, sequentially (host).
-__host__ __device__ __forceinline__ void plan_header(const BandPlan& p, int n_rows, int* hdr) {
+__host__ __device__ __forceinline__ void plan_header(const BandPlan& plan, int n_rows, int* hdr) {
+  const BandPlan p = plan_resolve(plan, n_rows);
   const int vsplit = plan_vsplit(p, n_rows);
   int gm = 1, gv = 1, gm2 = 0, gv2 = 0;
   plan_choose(plan_share(p, vsplit, 0), n_rows, &gm, &gv);
@@ -370,7 +389,8 @@ __host__ __device__ __forceinline__ void plan_header(const BandPlan& p, int n_ro
 #ifdef __CUDACC__
 // The same header by one CTA (the kernel that learns N calls it once); thread
 // 0 writes it.
-__device__ __forceinline__ void plan_write_header(const BandPlan& p, int n_rows, int* hdr, PlanScratch* sh) {
+__device__ __forceinline__ void plan_write_header(const BandPlan& plan, int n_rows, int* hdr, PlanScratch* sh) {
+  const BandPlan p = plan_resolve(plan, n_rows);
   const int vsplit = plan_vsplit(p, n_rows);
   int gm = 1, gv = 1, gm2 = 0, gv2 = 0;
   plan_choose_cta(plan_share(p, vsplit, 0), n_rows, &gm, &gv, sh);
@@ -393,6 +413,12 @@ __host__ __device__ __forceinline__ int hdr_word(const int* hdr, int i) {
 __host__ __device__ __forceinline__ int plan_max_slots(const BandPlan& p) {
   const int steps = cdiv(p.n_vt, plan_vc(p));
   int s = plan_unit_slots(p) * (p.G < steps ? p.G : steps);
+  if (p.adapt) {  // and as a single token group
+    const BandPlan q = plan_resolve(p, 0);
+    const int steps1 = cdiv(q.n_vt, plan_vc(q));
+    const int s1 = plan_unit_slots(q) * (q.G < steps1 ? q.G : steps1);
+    s = s1 > s ? s1 : s;
+  }
   if (p.G2 > 0) s += SPILL_UNIT_SLOTS * (p.G2 < p.n_vt ? p.G2 : p.n_vt);
   return s;
 }
@@ -410,11 +436,12 @@ struct TileIter {
   int vt, vt_end;  // its range in steps of vc v-tiles (the spill launch: v-tiles from vt0)
 
   // hdr: the workspace header the kernel that learns N wrote (HDR_*)
-  __host__ __device__ void init(const BandPlan& plan, const int* hdr, int runner_index) {
+  __host__ __device__ void init(const BandPlan& stored, const int* hdr, int runner_index) {
+    const int n_rows = hdr_word(hdr, HDR_N);
+    const BandPlan plan = plan_resolve(stored, n_rows);
     runner = runner_index;
     G = plan.G;
     mc = plan_mc(plan);
-    const int n_rows = hdr_word(hdr, HDR_N);
     n_mt = plan_runner_mts(plan, n_rows);
     const bool spill = plan.role == 1;
     const int vsplit = hdr_word(hdr, HDR_VSPLIT);

@@ -34,7 +34,8 @@
 // way cut the 8 x 2 x 32 bf16 LM head by ~11% in a diagnostic build in which
 // one of the two pairs skipped its head loads.
 //
-// Or the two pairs share token rows (the plan's vc = 2): they hold the same
+// Or the two pairs share token rows (the plan's vc = 2; windows of a single
+// token group take it on the device, see plan_resolve): they hold the same
 // token group and take the two v-tiles of each step of their vocabulary part
 // (v-tiles 2t and 2t + 1), each CTA loading its own head rows and a quarter
 // of its pair's token rows, multicast to the CTA of the same rank in the
@@ -347,11 +348,9 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   PairCtl* ctl = &tail->ctl;
   const uint32_t smem_base = smem_u32(smem);
 
-  // pairs per cluster (two share each head tile by multicast); quantised
-  // heads run without clusters
-  // pairs per cluster: two sharing head tiles (mc = 2) or token rows (vc = 2)
-  const int VC = QUANT ? 1 : plan_vc(a.plan);
-  const int MC = QUANT ? 1 : plan_mc(a.plan) * VC;
+  // pairs per cluster: two sharing head tiles (mc = 2) or token rows (vc = 2);
+  // quantised heads run without clusters
+  const int MC = QUANT ? 1 : plan_mc(a.plan) * plan_vc(a.plan);
   if constexpr (pair_cluster<HF>()) {
     // launched without its cluster there is no peer CTA to map or to pair
     // MMAs with: report and do nothing
@@ -367,7 +366,6 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   // half of the v-tile this CTA takes on its own
   const uint32_t rank = QUANT ? (blockIdx.x & 1u) : (crank & 1u);
   const int pp = static_cast<int>(crank >> 1);  // this pair's token group (vc = 1) or v-tile (vc = 2) in the runner
-  const int pp_mt = VC == 1 ? pp : 0;           // ... its token group within the runner's m-tiles
   const uint32_t lead = crank & ~1u;            // cluster rank of this pair's issuing CTA
   const uint32_t pair_mask = 3u << (2 * pp);    // both CTAs of this pair
   const uint32_t all_mask = (1u << (2 * MC)) - 1u;
@@ -425,6 +423,8 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   if (!spill) griddep_wait();
   if (!spill && a.plan.G2 > 0) griddep_launch_dependents();
   const int n_rows = hdr_word(a.n_rows, HDR_N);
+  const int VC = QUANT ? 1 : plan_vc(plan_resolve(a.plan, n_rows));
+  const int pp_mt = VC == 1 ? pp : 0;  // this pair's token group within the runner's m-tiles
   constexpr int BK = stage_k<HF>();
   constexpr int ACOLS = atom_cols<HF>();
   constexpr int NATOM = BK / ACOLS;
