@@ -168,6 +168,20 @@ int check_head(const bd_hidden* h, const bd_weight* w, int64_t rows, int variant
   return BD_OK;
 }
 
+// An E4M3 head: the pair kernel multiplies its codes directly on the 8-bit
+// tensor path, with the bf16 rows packed as two E4M3 terms (needs 16-byte
+// aligned code rows), at every window size. 64 x (4 + 1) verification rows
+// (d = 3584, V = 152064) take 233 us this way and 412 us with the codes decoded
+// to bf16 in the kernel, whose converter warps bound it.
+void choose_split(const bd_weight* w, int variant, Call* c) {
+  if (c->tc && w->dtype == BD_E4M3 && (variant == 0 || variant == 3) && env_int("BD_E4M3_SPLIT", 1, 0, 1) != 0 &&
+      aligned(w->data, 16) && w->ld % 16 == 0 && w->dim >= 16) {
+    c->pair = true;
+    c->split = true;
+    c->fused = false;
+  }
+}
+
 int check_args(const bd_hidden* h, const bd_weight* w, const bd_mask_state* ms, const bd_tau_grid* tg,
                int variant, Call* c) {
   if (!h || !w || !ms || !tg) return BD_ERR_NULL;
@@ -185,15 +199,7 @@ int check_args(const bd_hidden* h, const bd_weight* w, const bd_mask_state* ms, 
   if (ms->mask_token_id < -1 || ms->mask_token_id >= w->vocab) return BD_ERR_ARG;
   if (ms->mask_token_id >= 0 && w->vocab < 2) return BD_ERR_SHAPE;  // nothing left to predict
   if (P > 0 && (!ms->pos_masked || !ms->block_flags)) return BD_ERR_NULL;
-  // An E4M3 head on the commit step: the pair kernel multiplies its codes
-  // directly on the 8-bit tensor path, with the bf16 rows packed as two E4M3
-  // terms (needs 16-byte aligned code rows), at every window size.
-  if (c->tc && w->dtype == BD_E4M3 && (variant == 0 || variant == 3) && env_int("BD_E4M3_SPLIT", 1, 0, 1) != 0 &&
-      aligned(w->data, 16) && w->ld % 16 == 0 && w->dim >= 16) {
-    c->pair = true;
-    c->split = true;
-    c->fused = false;
-  }
+  choose_split(w, variant, c);
   c->P = P;
   c->n_seq = ms->n_seq;
   c->n_slots = ms->n_slots;
@@ -1020,7 +1026,7 @@ struct VerifyCall {
 };
 
 int check_verify(const bd_hidden* h, const bd_weight* w, const bd_draft* dr, const bd_eps_grid* eg, int variant,
-                 VerifyCall* vc) {
+                 VerifyCall* vc, bool allow_split = true) {
   if (!h || !w || !dr || !eg) return BD_ERR_NULL;
   if (!eg->eps || eg->E < 1 || eg->E > 31) return BD_ERR_TAU;
   for (int k = 0; k < eg->E; ++k)
@@ -1034,6 +1040,7 @@ int check_verify(const bd_hidden* h, const bd_weight* w, const bd_draft* dr, con
   if (const int rc = check_head(h, w, R, variant, &c)) return rc;
   if (R > 0 && !dr->draft) return BD_ERR_NULL;
   if (R > 0 && !aligned(dr->draft, 4)) return BD_ERR_ALIGN;
+  if (allow_split) choose_split(w, variant, &c);
   c.P = R;
   c.n_seq = dr->n_req;
   c.n_slots = 1;
@@ -1041,14 +1048,14 @@ int check_verify(const bd_hidden* h, const bd_weight* w, const bd_draft* dr, con
   c.n_blocks = dr->n_req;
   c.mask_id = -1;  // the target's full distribution
   c.T = eg->E;
-  c.ldc = h->ld;  // the rows are read in place
+  c.ldc = h->ld;  // the rows are read in place (two E4M3 terms of them with c.split)
   vc->n_req = dr->n_req;
   vc->n_draft = dr->n_draft;
   return BD_OK;
 }
 
 struct VerifyLayout {
-  size_t hdr, idx, draft_row, pm, ps, pa, pt, px, wq, total;
+  size_t hdr, idx, draft_row, pm, ps, pa, pt, px, hc, tsc, wq, total;
 };
 
 VerifyLayout make_verify_layout(const Call& c, const BandPlan& p) {
@@ -1070,6 +1077,8 @@ VerifyLayout make_verify_layout(const Call& c, const BandPlan& p) {
   l.pa = take(4 * slots * R, 256);
   l.pt = take(4 * slots * R, 256);
   l.px = take(4 * slots * R, 256);
+  l.hc = c.split ? take(2 * static_cast<size_t>(round_up(c.d, 16)) * R, 1024) : 0;
+  l.tsc = c.split ? take(4 * R, 256) : 0;
   l.wq = decoded_head(c) ? take(2 * static_cast<size_t>(c.ldq) * static_cast<size_t>(c.V), 1024) : 0;
   l.total = (off + 255) / 256 * 256;
   return l;
@@ -1090,11 +1099,26 @@ int run_verify(const VerifyCall& vc, const BandPlan& plan, const VerifyLayout& l
   float* px = reinterpret_cast<float*>(ws + lay.px);
   const int R = static_cast<int>(c.P);
 
-  int rc = cuda_status(bd::launch_prep_verify(draft->draft, vc.n_req, vc.n_draft, idx, draft_row, n_rows, plan, st));
+  bd::PrepVerifyArgs prep;
+  prep.draft = draft->draft;
+  prep.n_req = vc.n_req;
+  prep.n_draft = vc.n_draft;
+  prep.idx = idx;
+  prep.draft_row = draft_row;
+  prep.n_rows = n_rows;
+  prep.plan = plan;
+  prep.hidden = static_cast<const __nv_bfloat16*>(hidden->data);
+  prep.ld = c.ldh;
+  prep.d = static_cast<int>(c.d);
+  prep.hc = c.split ? ws + lay.hc : nullptr;
+  prep.ldc = ld_fp8_rows(c);
+  prep.tok_scale = c.split ? reinterpret_cast<float*>(ws + lay.tsc) : nullptr;
+  int rc = cuda_status(bd::launch_prep_verify(prep, c.split ? bd::ROWS_E4M3X2 : bd::ROWS_BF16, st));
   if (rc != BD_OK) return rc;
 
-  rc = launch_lmhead(c, plan, hidden, weight, hidden->data, c.ldh, ws + lay.wq, idx, n_rows, draft_row,
-                     Partials{pm, ps, pa, pt, px}, status, sm_count, ev_begin, ev_end, st);
+  rc = launch_lmhead(c, plan, hidden, weight, c.split ? prep.hc : hidden->data, c.split ? prep.ldc : c.ldh,
+                     ws + lay.wq, idx, n_rows, draft_row, Partials{pm, ps, pa, pt, px}, status, sm_count, ev_begin,
+                     ev_end, st, prep.tok_scale);
   if (rc != BD_OK) return rc;
 
   bd::VerifyArgs va;
@@ -1158,9 +1182,17 @@ int bd_verify_step(const bd_hidden* hidden, const bd_weight* weight, const bd_dr
   if (rc != BD_OK) return rc;
   BandPlan plan = make_plan(vc.c, ctx->sm_count, ctx->pairs, ctx->quads);
   VerifyLayout lay = make_verify_layout(vc.c, plan);
-  if (exec && exec->workspace && exec->workspace_bytes < lay.total && plan.adapt) {
-    plan.adapt = 0;  // as fit_layout
-    lay = make_verify_layout(vc.c, plan);
+  if (exec && exec->workspace && exec->workspace_bytes < lay.total) {
+    // as fit_layout; then without packed rows, the head decoded in the LM head
+    if (plan.adapt) {
+      plan.adapt = 0;
+      lay = make_verify_layout(vc.c, plan);
+    }
+    if (exec->workspace_bytes < lay.total && vc.c.split) {
+      if ((rc = check_verify(hidden, weight, draft, eps, variant, &vc, false)) != BD_OK) return rc;
+      plan = make_plan(vc.c, ctx->sm_count, ctx->pairs, ctx->quads);
+      lay = make_verify_layout(vc.c, plan);
+    }
   }
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {

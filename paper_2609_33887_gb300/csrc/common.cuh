@@ -115,8 +115,8 @@ __host__ __device__ __forceinline__ int plan_vc(const BandPlan& p) { return p.vc
 // group, sharing head tiles would leave the second pair multiplying zero rows:
 // the pairs share the group's rows and take two v-tiles instead. 8 x 2 x 32
 // windows with every other position resolved (N = 256, d = 2048, V = 151936),
-// LM head before and after: bf16 170 -> 115 us, E4M3 162 -> 101 us, W8A8
-// 104 -> 68 us; N = 128: 117 -> 100, 88 -> 59, 74 -> 57 us. With two groups
+// LM head before and after: bf16 170 -> 113 us, E4M3 162 -> 100 us, W8A8
+// 104 -> 68 us; N = 128: 117 -> 98, 88 -> 58, 74 -> 55 us. With two groups
 // (N = 257..512) sharing head tiles stays faster: 146 against 152 us a step at
 // N = 294 in bf16, 135 against 144 us with an E4M3 head.
 __host__ __device__ __forceinline__ BandPlan plan_resolve(const BandPlan& p, int n_rows) {

@@ -249,6 +249,8 @@ static_assert(stage_count<HF_W8A8, false>(160) == 7 && stage_count<HF_W8A8, fals
               "W8A8: seven 26 KB stages at NT = 160, five 32 KB stages at NT = 256");
 static_assert(stage_count<HF_E4M3X2, false>(160) == 5 && stage_count<HF_E4M3X2, false>(256) == 4,
               "two-term rows: five 36 KB stages at NT = 160, four 48 KB stages at NT = 256");
+static_assert(stage_count<HF_E4M3X2, true>(160) == 5 && stage_count<HF_E4M3X2, true>(256) == 4,
+              "two-term rows: the same stages on the verification path");
 static_assert(stage_count<HF_NVFP4, false>(160) == 4 && stage_count<HF_E4M3, false>(160) == 4 &&
                   stage_count<HF_NVFP4, true>(160) == 4 && stage_count<HF_E4M3, true>(160) == 4,
               "four operand stages at NT = 160 for quantised heads");
@@ -335,7 +337,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   constexpr bool QUANT = is_quant<HF>();
   constexpr bool W8A8 = HF == HF_W8A8;
   constexpr bool X2 = HF == HF_E4M3X2;
-  static_assert(!((W8A8 || X2) && VERIFY), "the 8-bit instantiations serve the commit step");
+  static_assert(!(W8A8 && VERIFY), "W8A8 serves the commit step");
   // commit step with a head decoded in the kernel: f16 operands (the decode
   // ends at f16), token rows pre-scaled by a power of two per row
   constexpr bool F16OPS = QUANT && !VERIFY;
@@ -794,7 +796,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
                   s[c] = 0.f;
                   t[c] = 0.f;
                 } else {
-                  const float dm = (m[c] - cm) * LOG2E;
+                  const float dm = (m[c] - cm) * k2[c];
                   const float f = ex2_approx(dm);
                   t[c] = f * fmaf(dm, s[c], t[c]);
                   s[c] *= f;
@@ -865,7 +867,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
           tail->w[ew].st.a[c * 32 + lane] = arg[c];
           if constexpr (VERIFY) {
             tail->w[ew].st.t[c * 32 + lane] = t[c];
-            tail->w[ew].st.x[c * 32 + lane] = lx[c];
+            tail->w[ew].st.x[c * 32 + lane] = TOKS ? lx[c] * ts[c] : lx[c];
           }
         }
       }
@@ -1035,8 +1037,9 @@ cudaError_t launch_lmhead_pair(const PairTokenMaps& tmH, const CUtensorMap& tmW,
       if (verify) return cudaErrorInvalidValue;
       return launch_pair<HF_W8A8, false>(tmH, tmW, q, lo, a, st);
     case HF_E4M3X2:
-      if (verify || tmLo == nullptr) return cudaErrorInvalidValue;
-      return launch_pair<HF_E4M3X2, false>(tmH, tmW, q, lo, a, st);
+      if (tmLo == nullptr) return cudaErrorInvalidValue;
+      return verify ? launch_pair<HF_E4M3X2, true>(tmH, tmW, q, lo, a, st)
+                    : launch_pair<HF_E4M3X2, false>(tmH, tmW, q, lo, a, st);
     case HF_E4M3:
       return verify ? launch_pair<HF_E4M3, true>(tmH, tmW, q, lo, a, st)
                     : launch_pair<HF_E4M3, false>(tmH, tmW, q, lo, a, st);

@@ -191,8 +191,69 @@ __device__ __forceinline__ void row_factors(float amax, float* up, float* scale)
   }
 }
 
+// Bytes between packed rows: ldc counts 16-bit elements, or bytes for the 8-bit formats.
+template <int FMT>
+__device__ __forceinline__ int64_t packed_row_bytes(int64_t ldc) {
+  return FMT == ROWS_BF16 || FMT == ROWS_F16_POW2 ? 2 * ldc : ldc;
+}
+
+// One warp packs the d elements of the bf16 row src into dst (16-byte aligned
+// rows of row_bytes; ROWS_E4M3X2: the lo terms lo_offset bytes after the hi
+// terms) and returns the row's token scale.
+template <int FMT>
+__device__ __forceinline__ float pack_row(const __nv_bfloat16* __restrict__ src, int d, uint8_t* __restrict__ dst,
+                                          int64_t lo_offset) {
+  const int lane = threadIdx.x & 31, nvec = d / 8;
+  const uint4* s4 = reinterpret_cast<const uint4*>(src);
+  if constexpr (FMT == ROWS_BF16) {
+    uint4* d4 = reinterpret_cast<uint4*>(dst);
+#pragma unroll 8
+    for (int v = lane; v < nvec; v += 32) d4[v] = __ldg(s4 + v);
+    for (int e = nvec * 8 + lane; e < d; e += 32) reinterpret_cast<__nv_bfloat16*>(dst)[e] = src[e];
+    return 1.f;
+  } else {
+    // rows of up to 32 * RC vectors (5120 bf16) are read once, into registers
+    constexpr int RC = 20;
+    const bool cached = nvec <= 32 * RC;
+    uint4 qc[RC];
+    float amax = 0.f;
+    if (cached) {
+#pragma unroll
+      for (int k = 0; k < RC; ++k) {
+        const int v = lane + 32 * k;
+        qc[k] = v < nvec ? __ldg(s4 + v) : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int k = 0; k < RC; ++k) amax = fmaxf(amax, amax8(qc[k]));
+    } else {
+#pragma unroll 4
+      for (int v = lane; v < nvec; v += 32) amax = fmaxf(amax, amax8(__ldg(s4 + v)));
+    }
+    for (int e = nvec * 8 + lane; e < d; e += 32) amax = fmaxf(amax, fabsf(__bfloat162float(src[e])));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    RowOut<FMT> out;
+    float scale;
+    row_factors<FMT>(amax, &out.up, &scale);
+    out.hi = dst;
+    out.lo = dst + lo_offset;
+    if (cached) {
+#pragma unroll
+      for (int k = 0; k < RC; ++k) {
+        const int v = lane + 32 * k;
+        if (v < nvec) out.store8(qc[k], v);
+      }
+    } else {
+#pragma unroll 4
+      for (int v = lane; v < nvec; v += 32) out.store8(__ldg(s4 + v), v);
+    }
+    for (int e = nvec * 8 + lane; e < d; e += 32) out.store1(__bfloat162float(src[e]), e);
+    return scale;
+  }
+}
+
 template <int FMT>  // the packed row format (ROWS_*); one instantiation per format
-__global__ void __launch_bounds__(PREP_THREADS) prep_rows_kernel(PrepArgs a) {
+__global__ void __launch_bounds__(PREP_THREADS, 2) prep_rows_kernel(PrepArgs a) {
   __shared__ int red[2][PREP_WARPS];
   __shared__ int rows_s[PREP_MAX_CHUNK];
   __shared__ PlanScratch plan_s;
@@ -249,58 +310,13 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_rows_kernel(PrepArgs a) {
   if (a.hidden == nullptr) return;
 
   // 2. pack the chunk's live rows
-  const int d = a.d, nvec = d / 8;
+  const int64_t row_bytes = packed_row_bytes<FMT>(a.ldc);
   for (int i = warp; i < local_total; i += PREP_WARPS) {
-    if (!index_ok(prefix + i, a.P, a.status)) continue;
-    const __nv_bfloat16* src = a.hidden + static_cast<int64_t>(rows_s[i]) * a.ld;
-    const uint4* s4 = reinterpret_cast<const uint4*>(src);
-    if constexpr (FMT == ROWS_BF16) {
-      __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(a.hc) + static_cast<int64_t>(prefix + i) * a.ldc;
-      uint4* d4 = reinterpret_cast<uint4*>(dst);
-#pragma unroll 8
-      for (int v = lane; v < nvec; v += 32) d4[v] = __ldg(s4 + v);
-      for (int e = nvec * 8 + lane; e < d; e += 32) dst[e] = src[e];
-    } else {
-      // rows of up to 32 * RC vectors (5120 bf16) are read once, into registers
-      constexpr int RC = 20;
-      const bool cached = nvec <= 32 * RC;
-      uint4 qc[RC];
-      float amax = 0.f;
-      if (cached) {
-#pragma unroll
-        for (int k = 0; k < RC; ++k) {
-          const int v = lane + 32 * k;
-          qc[k] = v < nvec ? __ldg(s4 + v) : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int k = 0; k < RC; ++k) amax = fmaxf(amax, amax8(qc[k]));
-      } else {
-#pragma unroll 4
-        for (int v = lane; v < nvec; v += 32) amax = fmaxf(amax, amax8(__ldg(s4 + v)));
-      }
-      for (int e = nvec * 8 + lane; e < d; e += 32) amax = fmaxf(amax, fabsf(__bfloat162float(src[e])));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-      // ldc counts bytes for the 8-bit formats, f16 elements for ROWS_F16_POW2
-      const int64_t row_bytes = FMT == ROWS_F16_POW2 ? 2 * a.ldc : a.ldc;
-      RowOut<FMT> out;
-      float scale;
-      row_factors<FMT>(amax, &out.up, &scale);
-      out.hi = static_cast<uint8_t*>(a.hc) + static_cast<int64_t>(prefix + i) * row_bytes;
-      out.lo = out.hi + static_cast<int64_t>(a.P) * row_bytes;
-      if (cached) {
-#pragma unroll
-        for (int k = 0; k < RC; ++k) {
-          const int v = lane + 32 * k;
-          if (v < nvec) out.store8(qc[k], v);
-        }
-      } else {
-#pragma unroll 4
-        for (int v = lane; v < nvec; v += 32) out.store8(__ldg(s4 + v), v);
-      }
-      for (int e = nvec * 8 + lane; e < d; e += 32) out.store1(__bfloat162float(src[e]), e);
-      if (lane == 0) a.tok_scale[prefix + i] = scale;
-    }
+    const int r = prefix + i;
+    if (!index_ok(r, a.P, a.status)) continue;
+    const float scale = pack_row<FMT>(a.hidden + static_cast<int64_t>(rows_s[i]) * a.ld, a.d,
+                                      static_cast<uint8_t*>(a.hc) + r * row_bytes, a.P * row_bytes);
+    if (FMT != ROWS_BF16 && lane == 0) a.tok_scale[r] = scale;
   }
 }
 
@@ -346,35 +362,45 @@ cudaError_t launch_prep_rows(const PrepArgs& args, int row_format, int sm_count,
 // ---------------------------------------------------------------------------
 // Verification rows need no compaction: every row is live. Row
 // r = q * (n_draft + 1) + i verifies draft token i of request q (i < n_draft);
-// the last row of a request verifies nothing.
+// the last row of a request verifies nothing. bf16 and NVFP4 heads read the
+// caller's rows in place (ROWS_BF16 here: nothing to pack); an E4M3 head on
+// the 8-bit path reads them as two E4M3 terms, packed by one warp per row.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(PREP_THREADS) prep_verify_kernel(const int32_t* __restrict__ draft, int n_req,
-                                                                   int n_draft, int* __restrict__ idx,
-                                                                   int* __restrict__ draft_row,
-                                                                   int* __restrict__ n_rows, BandPlan plan) {
+template <int FMT>
+__global__ void __launch_bounds__(PREP_THREADS, 2) prep_verify_kernel(PrepVerifyArgs a) {
   __shared__ PlanScratch plan_s;
   griddep_launch_dependents();
   griddep_wait();
-  const int R = n_req * (n_draft + 1);
+  const int D = a.n_draft, R = a.n_req * (D + 1);
   if (blockIdx.x == 0) {  // N and the plan for it
-    plan_write_header(plan, R, n_rows, &plan_s);
+    plan_write_header(a.plan, R, a.n_rows, &plan_s);
     return;
   }
-  const int step = (gridDim.x - 1) * PREP_THREADS;
-  for (int r = (blockIdx.x - 1) * PREP_THREADS + threadIdx.x; r < R; r += step) {
-    const int q = r / (n_draft + 1), i = r % (n_draft + 1);
-    idx[r] = r;
-    draft_row[r] = i < n_draft ? draft[q * n_draft + i] : -1;
+  const int cta = static_cast<int>(blockIdx.x) - 1, ctas = static_cast<int>(gridDim.x) - 1;
+  for (int r = cta * PREP_THREADS + threadIdx.x; r < R; r += ctas * PREP_THREADS) {
+    const int q = r / (D + 1), i = r % (D + 1);
+    a.idx[r] = r;
+    a.draft_row[r] = i < D ? a.draft[q * D + i] : -1;
+  }
+  if constexpr (FMT != ROWS_BF16) {
+    const int64_t row_bytes = packed_row_bytes<FMT>(a.ldc);
+    for (int r = cta * PREP_WARPS + static_cast<int>(threadIdx.x >> 5); r < R; r += ctas * PREP_WARPS) {
+      const float scale = pack_row<FMT>(a.hidden + static_cast<int64_t>(r) * a.ld, a.d,
+                                        static_cast<uint8_t*>(a.hc) + r * row_bytes, R * row_bytes);
+      if ((threadIdx.x & 31) == 0) a.tok_scale[r] = scale;
+    }
   }
 }
 
-cudaError_t launch_prep_verify(const int32_t* draft, int n_req, int n_draft, int* idx, int* draft_row, int* n_rows,
-                               const BandPlan& plan, cudaStream_t st) {
-  const int R = n_req * (n_draft + 1);
-  int grid = (R + PREP_THREADS - 1) / PREP_THREADS;
+cudaError_t launch_prep_verify(const PrepVerifyArgs& a, int row_format, cudaStream_t st) {
+  if (row_format != ROWS_BF16 && row_format != ROWS_E4M3X2) return cudaErrorInvalidValue;
+  const int R = a.n_req * (a.n_draft + 1);
+  const int rows = row_format == ROWS_BF16 ? PREP_THREADS : PREP_WARPS;  // per CTA
+  int grid = (R + rows - 1) / rows;
   if (grid < 1) grid = 1;
   if (grid > 1024) grid = 1024;
-  return launch_behind(prep_verify_kernel, 1 + grid, st, draft, n_req, n_draft, idx, draft_row, n_rows, plan);
+  return row_format == ROWS_BF16 ? launch_behind(prep_verify_kernel<ROWS_BF16>, 1 + grid, st, a)
+                                 : launch_behind(prep_verify_kernel<ROWS_E4M3X2>, 1 + grid, st, a);
 }
 
 // ---------------------------------------------------------------------------

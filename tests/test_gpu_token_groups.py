@@ -101,3 +101,20 @@ def test_verify_step(head, V, n_req):
     clear = (p[:, None] - bar).abs() > 4e-3
     assert torch.equal(bits[clear], (p[:, None] > bar)[clear])
 
+
+def test_verify_with_the_workspace_of_rows_read_in_place(monkeypatch):
+    # an E4M3 head's rows are packed in the workspace; one that has no room for
+    # them is taken as well (the head is then decoded in the kernel)
+    n_req, D, d, V = 6, 4, 336, 700
+    h, w, scale, logit = make("e4m3", n_req * (D + 1), V, d, 3)
+    draft = logit.argmax(1).view(n_req, D + 1)[:, :D].int().reshape(-1).contiguous()
+    monkeypatch.setenv("BD_E4M3_SPLIT", "0")
+    least = bdc.bd_verify_workspace_size(h, w, scale, draft, n_req, D, [0.3])
+    monkeypatch.delenv("BD_E4M3_SPLIT")
+    want = bdc.verify_step(h, w, draft, n_req, D, [0.3], weight_scale=scale)
+    for size in (least, least + 64 * 1024):
+        ws = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+        ws = ws[(-ws.data_ptr()) % 256:][:size]
+        got = bdc.verify_step(h, w, draft, n_req, D, [0.3], weight_scale=scale, workspace=ws)
+        assert torch.equal(got["tokens"], want["tokens"]) and torch.equal(got["accepted"], want["accepted"])
+        assert float((got["p_draft"] - want["p_draft"]).abs().max()) < 4e-4
