@@ -86,6 +86,7 @@ struct Call {
   int64_t ldq;      // decoded e4m3 head (bf16), elements
   bool fused;       // pair kernel decodes an E4M3 / NVFP4 head itself (no bf16 copy)
   bool fp8_act = false;  // W8A8: token rows quantised to E4M3, kind::f8f6f4 MMAs on the E4M3 head
+  bool verify = false;   // verification rows (bd_verify_step)
   bool split = false;    // W8A16 on the 8-bit path: bf16 rows as two E4M3 terms times the E4M3 head
 };
 
@@ -240,7 +241,7 @@ BandPlan make_plan(const Call& c, int sm_count, int pairs, int quads) {
   BandPlan p{};
   p.mc = 1;
   if (c.pair) {
-    p.BM = 0;  // token groups derived from N on the device
+    p.BM = bd::BM_PAIR;  // token groups derived from N on the device
     p.BN = 256;
     p.G = pairs;
     p.cpu = 2;
@@ -283,9 +284,11 @@ BandPlan make_plan(const Call& c, int sm_count, int pairs, int quads) {
     p.G = sm_count;
     p.cpu = 1;
   } else {
-    p.BM = bd::SIMT_BM;
-    p.BN = bd::SIMT_BN;
-    p.G = 2 * sm_count;
+    // tiles of 128 entries unless the window (in groups of 96 rows) then has
+    // fewer than two tiles per SM
+    p.BM = bd::BM_SIMT;
+    p.BN = (c.P + 95) / 96 * ((c.V + bd::SIMT_BN - 1) / bd::SIMT_BN) < 2 * sm_count ? bd::SIMT_BN_SMALL : bd::SIMT_BN;
+    p.G = (c.verify ? bd::SIMT_CTAS_VERIFY : bd::SIMT_CTAS) * sm_count;
     p.cpu = 1;
   }
   // bands: GM derived on the device from the head and row bytes (0), or fixed
@@ -328,15 +331,20 @@ Layout make_layout(const Call& c, const BandPlan& p) {
   return l;
 }
 
-// The plan and layout for a workspace of `bytes`: the device's choice between
-// the cluster layouts needs up to twice the partial slots, and is left out
-// where they do not fit.
-Layout fit_layout(const Call& c, BandPlan* p, size_t bytes) {
+// A plan with fewer partial slots, for a workspace that does not hold those of
+// *p (true if it changed): without the device's choice between the cluster
+// layouts, and the SIMT kernel on fewer runners.
+bool shrink_plan(const Call& c, int sm_count, BandPlan* p) {
+  const int slots = plan_max_slots(*p);
+  p->adapt = 0;
+  if (!c.tc) p->G = static_cast<int>(std::min<int64_t>(2 * sm_count, (c.V + 63) / 64));
+  return plan_max_slots(*p) < slots;
+}
+
+// The plan and layout for a workspace of `bytes`.
+Layout fit_layout(const Call& c, BandPlan* p, int sm_count, size_t bytes) {
   Layout l = make_layout(c, *p);
-  if (l.total > bytes && p->adapt) {
-    p->adapt = 0;
-    l = make_layout(c, *p);
-  }
+  if (l.total > bytes && shrink_plan(c, sm_count, p)) l = make_layout(c, *p);
   return l;
 }
 
@@ -705,7 +713,7 @@ int bd_commit_step_ex(const bd_hidden* hidden, const bd_weight* weight, const bd
   rc = device_ctx(&ctx);
   if (rc != BD_OK) return rc;
   BandPlan plan = make_plan(c, ctx->sm_count, ctx->pairs, ctx->quads);
-  const Layout lay = fit_layout(c, &plan, exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX);
+  const Layout lay = fit_layout(c, &plan, ctx->sm_count, exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX);
 
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {
@@ -760,7 +768,7 @@ int bd_lmhead_partials(const bd_hidden* hidden, const bd_weight* shard, int64_t 
   rc = device_ctx(&ctx);
   if (rc != BD_OK) return rc;
   BandPlan plan = make_plan(c, ctx->sm_count, ctx->pairs, ctx->quads);
-  const Layout lay = fit_layout(c, &plan, exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX);
+  const Layout lay = fit_layout(c, &plan, ctx->sm_count, exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX);
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {
     if (exec->workspace_bytes < lay.total) return BD_ERR_WORKSPACE;
@@ -972,7 +980,7 @@ extern "C" int bd_commit_step_static(const bd_hidden* hidden, const bd_weight* w
   rc = static_ctx(&sctx);
   if (rc != BD_OK) return rc;
   BandPlan plan = make_plan(c, sctx->sm_count, sctx->pairs, sctx->quads);
-  const Layout lay = fit_layout(c, &plan, BD_STATIC_SCRATCH_BYTES);
+  const Layout lay = fit_layout(c, &plan, sctx->sm_count, BD_STATIC_SCRATCH_BYTES);
   if (lay.total > BD_STATIC_SCRATCH_BYTES) return BD_ERR_WORKSPACE;
 
   uint8_t* ws = sctx->scratch;
@@ -1047,6 +1055,7 @@ int check_verify(const bd_hidden* h, const bd_weight* w, const bd_draft* dr, con
   c.L = dr->n_draft + 1;
   c.n_blocks = dr->n_req;
   c.mask_id = -1;  // the target's full distribution
+  c.verify = true;
   c.T = eg->E;
   c.ldc = h->ld;  // the rows are read in place (two E4M3 terms of them with c.split)
   vc->n_req = dr->n_req;
@@ -1184,10 +1193,7 @@ int bd_verify_step(const bd_hidden* hidden, const bd_weight* weight, const bd_dr
   VerifyLayout lay = make_verify_layout(vc.c, plan);
   if (exec && exec->workspace && exec->workspace_bytes < lay.total) {
     // as fit_layout; then without packed rows, the head decoded in the LM head
-    if (plan.adapt) {
-      plan.adapt = 0;
-      lay = make_verify_layout(vc.c, plan);
-    }
+    if (shrink_plan(vc.c, ctx->sm_count, &plan)) lay = make_verify_layout(vc.c, plan);
     if (exec->workspace_bytes < lay.total && vc.c.split) {
       if ((rc = check_verify(hidden, weight, draft, eps, variant, &vc, false)) != BD_OK) return rc;
       plan = make_plan(vc.c, ctx->sm_count, ctx->pairs, ctx->quads);

@@ -65,7 +65,7 @@ constexpr float FUSED_SHIFT_LIMIT = 2048.f;
 // and merge kernels read.
 // -------------------------------------------------------------------------
 struct BandPlan {
-  int BM;         // rows per m-tile; 0 = derived from N (token groups of the pair kernel)
+  int BM;         // rows per m-tile; derived from N when BM_PAIR or BM_SIMT
   int BN;         // vocabulary entries per v-tile
   int GM;         // m-tiles per band when > 0 (clamped to 1..n_mt); 0 = chosen with gv
   int G;          // runners that can run at once (CTAs, CTA pairs or clusters)
@@ -82,6 +82,10 @@ struct BandPlan {
   int spill_pct;  // a spill pair's time per tile against a cluster pair's, in percent (0: 100)
   int role;       // 0: the main launch; 1: the spill launch (single pairs, the last v-tiles)
 };
+
+// Values of BandPlan::BM: rows per m-tile derived from N
+constexpr int BM_PAIR = 0;   // the pair kernel's token groups
+constexpr int BM_SIMT = -2;  // simt_group_rows
 
 // Words of the workspace header (int32) the kernel that learns N writes for
 // the LM-head and merge kernels: N, the partial slots per row over all
@@ -104,8 +108,29 @@ __host__ __device__ __forceinline__ int pair_group_rows(int n_rows) {
   return cdiv(cdiv(n_rows, groups), 32) * 32;
 }
 
+// Rows per group of the SIMT kernel, at most 96, equal sizes rounded up to a
+// multiple of 8 (of 16 above 64). Up to 64 groups, of the four fewest group
+// counts the one whose rounds of tiles times rows cost least, the fewer groups
+// on a tie (77 rows: one group of 80, LM head 223 us against 240 us as two of
+// 40; 256 rows: four of 64, 684 us against 801 us as three of 96).
+__host__ __device__ __forceinline__ int simt_group_rows(const BandPlan& p, int n_rows) {
+  if (n_rows <= 0) return 8;
+  const int g0 = cdiv(n_rows, 96);
+  int best = 0, best_cost = 0;
+  for (int g = g0; g < (g0 <= 64 ? g0 + 4 : g0 + 1); ++g) {
+    int rows = cdiv(n_rows, g);
+    rows = rows <= 64 ? cdiv(rows, 8) * 8 : cdiv(rows, 16) * 16;
+    const int cost = cdiv(g * p.n_vt, p.G) * rows;  // 32 bits: g <= 67, n_vt <= 2^23
+    if (best == 0 || cost < best_cost) {
+      best = rows;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 __host__ __device__ __forceinline__ int plan_bm(const BandPlan& p, int n_rows) {
-  return p.BM > 0 ? p.BM : pair_group_rows(n_rows);
+  return p.BM > 0 ? p.BM : p.BM == BM_SIMT ? simt_group_rows(p, n_rows) : pair_group_rows(n_rows);
 }
 
 __host__ __device__ __forceinline__ int plan_mc(const BandPlan& p) { return p.mc > 1 ? p.mc : 1; }

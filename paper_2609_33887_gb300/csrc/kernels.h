@@ -145,8 +145,10 @@ struct SimtArgs {
   float* part_t = nullptr;
   float* part_x = nullptr;
 };
-constexpr int SIMT_BM = 32;
-constexpr int SIMT_BN = 64;
+constexpr int SIMT_BN = 128;       // vocabulary entries per tile
+constexpr int SIMT_BN_SMALL = 32;  // ... where those would leave most SMs without one
+// CTAs per SM (plan.G = this times the SMs; plan.BM = BM_SIMT)
+constexpr int SIMT_CTAS = 3, SIMT_CTAS_VERIFY = 2;
 cudaError_t launch_lmhead_simt(const SimtArgs& a, cudaStream_t st);
 
 // a3+a4: merge of the partials per row, then the threshold commit with the
