@@ -387,7 +387,7 @@ LEVERS = {
     # key: (workload, description of the LM-head path and what bounds it)
     "nvfp4": ("b8x2x32_d2048_v151936_nvfp4",
               "codes streamed by TMA and decoded exactly to f16 inside the LM-head kernel (f16 MMA, token rows "
-              "scaled by a power of two per row); bound: the converter warps"),
+              "scaled by a power of two per row); bound: the converter warps' chain per stage"),
     "e4m3": ("b8x2x32_d2048_v151936_e4m3",
              "W8A16 on the 8-bit tensor path: E4M3 codes read by TMA straight into the MMA operand; each bf16 row "
              "packed as two E4M3 terms (exact above 2^-10 of the row's largest), both multiplied by the head "
@@ -537,9 +537,8 @@ def masked_count(wl_host):
 
 def lmhead_launches(r):
     """LM-head launches per step: the library's kernel count less compaction,
-    merge and the head decode where a bf16 copy is made."""
-    decoded = r.cfg.weight_dtype == "nvfp4" and r.cfg.P > 8192
-    return launches_per_step(r) - 2 - (1 if decoded else 0)
+    merge (no workload's head is decoded to a bf16 copy)."""
+    return launches_per_step(r) - 2
 
 
 def launches_per_step(r):
@@ -547,7 +546,7 @@ def launches_per_step(r):
     reports them for its arguments (bd_step_kernels): compaction + row packing,
     the decode of a quantised head where a bf16 copy is made, the LM head (one
     launch, or two where spill pairs run beside clusters of two CTA pairs),
-    merge + commit. The counts reset is a runtime memset, not a kernel."""
+    merge + commit. The compaction kernel clears the counts."""
     n = r.kernels_per_step
     if n <= 0:
         raise RuntimeError(f"bd_step_kernels: {n}")

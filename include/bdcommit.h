@@ -105,15 +105,16 @@ typedef struct {
  *   ld * element size (bytes for BD_NVFP4) a multiple of 16.
  *   Both quantised formats decode exactly to bf16. A BD_E4M3 head on the
  *   commit step is read as it is by the 8-bit tensor path of the CTA-pair
- *   kernel at every window size (see bd_exec.variant), with no copy. For the
- *   other cases, on the CTA-pair kernel (windows up to 8192 positions) the
- *   codes are decoded inside the kernel, so the workspace holds no bf16 copy
- *   of the head, when a row holds at least 16 bytes of codes and, for
- *   BD_NVFP4, `block_scale` is 16-byte aligned with block_ld a multiple of
- *   16; otherwise the head is first decoded into a bf16 copy in the
- *   workspace (bd_workspace_size accounts for it). The environment variables
- *   BD_E4M3_SPLIT=0 (no 8-bit path) and BD_FUSED_DECODE=0 (no decode in the
- *   kernel) select the other paths. */
+ *   kernel at every window size (see bd_exec.variant), with no copy; so it is
+ *   for verification, whose rows are then packed in the workspace (a caller's
+ *   workspace without room for them is taken too, the codes being decoded as
+ *   below). For the other cases the CTA-pair kernel decodes the codes itself,
+ *   so the workspace holds no bf16 copy of the head, when a row holds at least
+ *   16 bytes of codes and, for BD_NVFP4, `block_scale` is 16-byte aligned with
+ *   block_ld a multiple of 16; otherwise the head is first decoded into a bf16
+ *   copy in the workspace (bd_workspace_size accounts for it). The environment
+ *   variables BD_E4M3_SPLIT=0 (no 8-bit path) and BD_FUSED_DECODE=0 (no decode
+ *   in the kernel) select the other paths. */
 typedef struct {
   const void* data;
   int32_t dtype;
@@ -165,11 +166,11 @@ typedef struct {
  *                     for timing it alone.
  *   variant         : 0 = automatic: the CTA-pair tensor-core kernel for BF16
  *                     heads at every window size and for E4M3 heads with
- *                     16-byte aligned rows (see below); NVFP4 heads (and E4M3
- *                     heads the 8-bit path cannot read) on the CTA-pair kernel
- *                     up to 8192 window positions and the one-CTA kernel on a
- *                     decoded bf16 copy above; the fp32 SIMT kernel for F32
- *                     heads. 1 = force the fp32-FMA SIMT LM-head kernel; 2 =
+ *                     16-byte aligned rows (see below), and for NVFP4 heads whose
+ *                     codes and block scales it can read as stored; quantised
+ *                     heads it cannot read so on the CTA-pair kernel up to 8192
+ *                     window positions and the one-CTA kernel above, on a decoded
+ *                     bf16 copy; the fp32 SIMT kernel for F32 heads. 1 = force the fp32-FMA SIMT LM-head kernel; 2 =
  *                     force the one-CTA tensor-core kernel (tokens on the MMA M
  *                     side); 3 = force the CTA-pair tensor-core kernel
  *                     (vocabulary on the M side). 2 and 3 need BF16 hidden
@@ -266,8 +267,10 @@ int bd_plan_header(const bd_hidden* hidden, const bd_weight* weight, const bd_ma
  * the work is done, never what is computed):
  *   BD_E4M3_SPLIT=0      E4M3 heads not on the 8-bit path (see bd_exec.variant)
  *   BD_FUSED_DECODE=0    quantised heads decoded to a bf16 copy, not in the kernel
- *   BD_PAIR_MAX_P=n      the automatic choice takes the CTA-pair kernel for NVFP4
- *                        heads up to n window positions (default 8192)
+ *   BD_PAIR_MAX_P=n      the automatic choice takes the CTA-pair kernel for
+ *                        quantised heads off the 8-bit path up to n window
+ *                        positions (default: always for heads decoded in the
+ *                        kernel, 8192 on a decoded copy)
  *   BD_PAIR_MC=1|2       single CTA pairs, or clusters of two pairs sharing each
  *                        head tile by multicast (default: clusters for windows of
  *                        at most 512 positions or more than 256 MiB of packed rows)

@@ -148,24 +148,27 @@ int check_head(const bd_hidden* h, const bd_weight* w, int64_t rows, int variant
   c->hdt = hdt;
   c->wdt = wdt;
   c->tc = tc;
+  // the pair kernel reads E4M3 / NVFP4 codes (and block scales) with TMA when
+  // their rows start on 16-byte boundaries; otherwise the head is decoded to a
+  // bf16 copy first
+  const bool quant_head = wdt == BD_E4M3 || wdt == BD_NVFP4;
+  const bool readable = quant_head && env_int("BD_FUSED_DECODE", 1, 0, 1) != 0 && aligned(w->data, 16) &&
+                        w->ld % 16 == 0 && (wdt == BD_NVFP4 ? (w->dim + 1) / 2 : w->dim) >= 16 &&
+                        (wdt != BD_NVFP4 || (aligned(w->block_scale, 16) && w->block_ld % 16 == 0));
   // automatic choice: the CTA-pair kernel (vocabulary on M, token dimension
   // padded only to a multiple of 32, 256 x 256 tiles per pair at large
-  // windows) for bf16 heads at every size; heads decoded in the kernel by its
-  // converter warps only while the window is small (at large windows the
-  // one-CTA kernel on a decoded bf16 copy keeps the tensor pipe busier)
-  const bool quant_head = wdt == BD_E4M3 || wdt == BD_NVFP4;
-  c->pair = tc && (variant == 3 ||
-                   (variant == 0 && (!quant_head || rows <= env_int("BD_PAIR_MAX_P", 8192, 0, 1 << 30))));
+  // windows) for every head it reads as stored (NVFP4, d = 2048, V = 151936:
+  // 3.17 against 3.49 ms a step at 9000 positions and 5.72 against 5.92 ms at
+  // 16384 with the one-CTA kernel on a decoded bf16 copy, which costs 0.2 ms);
+  // on a decoded copy only while the window is small (at large windows the
+  // one-CTA kernel keeps the tensor pipe busier)
+  const int max_p = env_int("BD_PAIR_MAX_P", readable ? 1 << 30 : 8192, 0, 1 << 30);
+  c->pair = tc && (variant == 3 || (variant == 0 && (!quant_head || rows <= max_p)));
   c->ldh = h->ld;
   c->ldw = w->ld;
   c->ldc = round_up(c->d, 8);
   c->ldq = round_up(c->d, 8);
-  // the pair kernel reads E4M3 / NVFP4 codes (and block scales) with TMA when
-  // their rows start on 16-byte boundaries; otherwise the head is decoded to a
-  // bf16 copy first
-  c->fused = c->pair && (wdt == BD_E4M3 || wdt == BD_NVFP4) && env_int("BD_FUSED_DECODE", 1, 0, 1) != 0 &&
-             aligned(w->data, 16) && w->ld % 16 == 0 && (wdt == BD_NVFP4 ? (w->dim + 1) / 2 : w->dim) >= 16 &&
-             (wdt != BD_NVFP4 || (aligned(w->block_scale, 16) && w->block_ld % 16 == 0));
+  c->fused = c->pair && readable;
   return BD_OK;
 }
 
@@ -241,7 +244,7 @@ BandPlan make_plan(const Call& c, int sm_count, int pairs, int quads) {
   BandPlan p{};
   p.mc = 1;
   if (c.pair) {
-    p.BM = bd::BM_PAIR;  // token groups derived from N on the device
+    p.BM = c.fused ? bd::BM_QUANT : bd::BM_PAIR;  // token groups derived from N on the device
     p.BN = 256;
     p.G = pairs;
     p.cpu = 2;

@@ -65,7 +65,7 @@ constexpr float FUSED_SHIFT_LIMIT = 2048.f;
 // and merge kernels read.
 // -------------------------------------------------------------------------
 struct BandPlan {
-  int BM;         // rows per m-tile; derived from N when BM_PAIR or BM_SIMT
+  int BM;         // rows per m-tile; derived from N when 0 (pair_group_rows), BM_QUANT or BM_SIMT
   int BN;         // vocabulary entries per v-tile
   int GM;         // m-tiles per band when > 0 (clamped to 1..n_mt); 0 = chosen with gv
   int G;          // runners that can run at once (CTAs, CTA pairs or clusters)
@@ -84,8 +84,10 @@ struct BandPlan {
 };
 
 // Values of BandPlan::BM: rows per m-tile derived from N
-constexpr int BM_PAIR = 0;   // the pair kernel's token groups
-constexpr int BM_SIMT = -2;  // simt_group_rows
+constexpr int BM_PAIR = 0;    // the pair kernel's token groups
+constexpr int BM_QUANT = -1;  // ... with a head decoded in the kernel: groups of at most QUANT_GROUP rows
+constexpr int BM_SIMT = -2;   // simt_group_rows
+constexpr int QUANT_GROUP = 192;
 
 // Words of the workspace header (int32) the kernel that learns N writes for
 // the LM-head and merge kernels: N, the partial slots per row over all
@@ -101,10 +103,10 @@ enum : int {
 __host__ __device__ __forceinline__ int cdiv(int a, int b) { return (a + b - 1) / b; }
 
 // Token-group size of the pair kernel for N rows: the fewest groups of at most
-// 256 rows, equal sizes rounded up to a multiple of 32 (16 rows per CTA).
-__host__ __device__ __forceinline__ int pair_group_rows(int n_rows) {
+// `most` rows, equal sizes rounded up to a multiple of 32 (16 rows per CTA).
+__host__ __device__ __forceinline__ int pair_group_rows(int n_rows, int most = 256) {
   if (n_rows <= 0) return 32;
-  const int groups = cdiv(n_rows, 256);
+  const int groups = cdiv(n_rows, most);
   return cdiv(cdiv(n_rows, groups), 32) * 32;
 }
 
@@ -130,7 +132,10 @@ __host__ __device__ __forceinline__ int simt_group_rows(const BandPlan& p, int n
 }
 
 __host__ __device__ __forceinline__ int plan_bm(const BandPlan& p, int n_rows) {
-  return p.BM > 0 ? p.BM : p.BM == BM_SIMT ? simt_group_rows(p, n_rows) : pair_group_rows(n_rows);
+  return p.BM > 0           ? p.BM
+         : p.BM == BM_SIMT  ? simt_group_rows(p, n_rows)
+         : p.BM == BM_QUANT ? pair_group_rows(n_rows, QUANT_GROUP)
+                            : pair_group_rows(n_rows);
 }
 
 __host__ __device__ __forceinline__ int plan_mc(const BandPlan& p) { return p.mc > 1 ? p.mc : 1; }
@@ -656,6 +661,19 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
   return ok;
 }
 
+// Whether the phase of parity `parity` has completed, without waiting for it.
+__device__ __forceinline__ uint32_t mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok;
+}
+
 // Single-thread bounded wait for the phase of parity `parity` to complete.
 // Returns false (and raises the CTA's abort flag) after WAIT_LIMIT_NS, or as
 // soon as another role of the CTA has raised the abort flag.
@@ -703,24 +721,16 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
   }
 }
 
-// Orders this thread's generic-proxy writes to shared memory before later
-// async-proxy accesses (TMA, tcgen05.mma operand reads) of the same memory.
-__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
 __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
   uint4 v;
   asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
   return v;
 }
 
-__device__ __forceinline__ uint32_t ld_shared_u16(uint32_t addr) {
-  uint16_t v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+__device__ __forceinline__ uint32_t ld_shared_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
   return v;
-}
-
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
 // Two E2M1 codes (low nibble: the lower element) -> f16x2 (lower element in the low half); exact.
@@ -913,6 +923,22 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Store 32 consecutive 32-bit columns of this thread's TMEM lane (32x32b
+// shape, x32 repeat); tmem_st_wait waits for the thread's stores to complete.
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};" ::"r"(r[0]),
+      "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+      "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
+      "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),
+      "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(taddr)
+      : "memory");
+}
+
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 // ---- programmatic dependent launch ------------------------------------------
 // Blocks until the grid this one depends on has completed and its writes are
 // visible (a no-op when the launch carries no programmatic dependency).
@@ -947,9 +973,14 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
   return r;
 }
 
-// Arrive once on an mbarrier given by its shared::cluster address (possibly in the peer CTA).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+// Arrive once on an mbarrier given by its shared::cluster address (possibly in
+// the peer CTA) without releasing the thread's memory accesses: it orders
+// tensor-memory accesses that tcgen05.fence::before_thread_sync precedes
+// (waited-for tcgen05.ld / tcgen05.st), with tcgen05.fence::after_thread_sync
+// behind the wait. The releasing form costs a cluster-scope fence, about 900
+// cycles of the arriving warp.
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
 // 2-D tiled load into this CTA's shared memory whose completion is counted on
@@ -999,6 +1030,19 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, 
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// The same with A in the tensor memory of both CTAs: row i of this CTA's 128
+// in lane i, two 16-bit elements per 32-bit column (16 elements, 8 columns per
+// instruction).
+__device__ __forceinline__ void umma_f16_pair_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                                 uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 

@@ -72,17 +72,30 @@
 // E4M3 products are exact in fp32.
 //
 // Heads decoded in the kernel (HF = HF_E4M3, HF_NVFP4: the precision levers):
-// HBM carries the stored head only. A raw-code producer warp streams this
-// CTA's head codes (and NVFP4 block scales) with TMA into a raw ring, and
-// eight converter warps decode them exactly into the operand tile of each
-// 64-column stage, in its 128-byte-swizzled layout: f16 on the commit step
-// (the token rows then come as f16 scaled by a power of two per row, undone
-// on the logits like W8A8's scales), bf16 for verification. Each CTA
-// multiplies its 128 head rows by all NT token rows with cta_group::1 MMAs,
-// so converters signal only their own CTA; the operand stage is full when
-// its eight converter warps have arrived and the token rows' bytes have
-// landed. E4M3 raw stages hold 128 columns of d, NVFP4 raw stages 256 (128
-// bytes of codes per row either way); 480 threads.
+// HBM carries the stored head only. A raw-code producer warp of each CTA
+// streams its head codes (and NVFP4 block scales) with TMA into a raw ring,
+// and twelve converter warps decode them exactly, a vocabulary row per thread,
+// straight into the tensor memory the pair's MMAs read their A operand from
+// (two tcgen05.st of 32 columns, 64 16-bit elements each, per warp and stage):
+// f16 on the commit step (the token rows then come as f16 scaled by a power of
+// two per row, undone on the logits like W8A8's scales), bf16 for
+// verification. Sets of four converter warps take the 128-column stages in
+// turn; each warp signals the issuing CTA's full barrier of the stage, which
+// counts the token rows' bytes too. E4M3 raw stages hold 128 columns of d,
+// NVFP4 raw stages 256 (128 bytes of codes per row either way). Two
+// accumulators of up to 192 columns leave room for the A stages, so token
+// groups hold at most 192 rows; 608 threads.
+//
+// What bounds these heads is the converters' chain of latencies per stage, not
+// the conversion (164 cycles per 64 columns if nothing else ran) nor the MMAs.
+// 294 rows, d = 2048, V = 151936, NVFP4: 123 us, 16 rows 62 us. Decoding into
+// shared memory with one CTA per half v-tile took 208 and 98 us: its chain had
+// the operand stores, a proxy fence and the token rows of a whole group in
+// shared memory besides. With A in tensor memory it went 145 us at 16 rows
+// with a releasing arrive at the peer's barrier (a cluster-scope fence of about
+// 900 cycles each), 80 us with the relaxed one, 75 us with one barrier per
+// 128-column stage, and 62 us with a whole stage per visit of a set instead of
+// 64 columns of it.
 #include <atomic>
 #include <cstring>
 
@@ -98,12 +111,6 @@ template <int HF>
 __host__ __device__ constexpr bool is_quant() {
   return HF == HF_E4M3 || HF == HF_NVFP4;
 }
-// Instantiations that issue cta_group::2 MMAs and must run as clusters of 2
-// (the heads decoded in the kernel run one CTA per half v-tile instead).
-template <int HF>
-__host__ __device__ constexpr bool pair_cluster() {
-  return !is_quant<HF>();
-}
 // E4M3 head codes read by TMA straight into the MMA operand (8-bit atoms)
 template <int HF>
 __host__ __device__ constexpr bool is_8bit() {
@@ -114,13 +121,9 @@ template <int HF>
 __host__ __device__ constexpr int b_terms() {
   return HF == HF_E4M3X2 ? 2 : 1;
 }
-// columns of d per operand stage: two 64-column 16-bit swizzle atoms for bf16
-// heads; one 128-column 8-bit atom for W8A8; one 16-bit atom for heads decoded
-// in the kernel, whose small stages leave room for a deep raw ring
-template <int HF>
-__host__ __device__ constexpr int stage_k() {
-  return is_quant<HF>() ? 64 : 128;
-}
+// columns of d per operand stage: two 64-column 16-bit swizzle atoms, or one
+// 128-column 8-bit atom
+constexpr int STAGE_K = 128;
 // columns of one 128-byte swizzle atom
 template <int HF>
 __host__ __device__ constexpr int atom_cols() {
@@ -133,11 +136,25 @@ constexpr uint32_t TMEM_COLS = 512;  // two accumulators of up to 256 columns, o
 constexpr int MAX_ACC = 3;
 constexpr int EPI_WARPS = 4;  // epilogue warps of the bf16 and decoded-head instantiations
 constexpr int TR = 34;  // padded row of the transpose buffers: 8-byte aligned rows, conflict-free column reads
-constexpr int MAX_CHUNKS = 8;
+// 32-column chunks of a token group
+template <int HF>
+__host__ __device__ constexpr int max_chunks() {
+  return is_quant<HF>() ? QUANT_GROUP / 32 : 8;
+}
 constexpr int MAX_RAW = 8;
-constexpr int QUANT_STAGES = 4;  // operand stages next to the raw ring (quantised heads)
-constexpr int CONV_WARPS = 8;                            // converter warps 6..13 (quantised heads)
-constexpr int CONV_THREADS = CONV_WARPS * 32;
+constexpr int MIN_RAW = 7;  // raw stages the token ring leaves room for (quantised heads)
+constexpr int QUANT_STAGES = 4;  // operand stages at most (quantised heads)
+// Decoded A stages in tensor memory (quantised heads), 64 columns of 16-bit
+// pairs each, written in parts of 32, behind two accumulators of NT columns: as
+// many as fit.
+constexpr uint32_t A_COLS = STAGE_K / 2;
+constexpr int PARTS = 2;                       // parts of a stage
+constexpr int PART_K = STAGE_K / PARTS;        // columns of d per part
+__host__ __device__ constexpr int a_stages(int nt) {
+  return (static_cast<int>(TMEM_COLS) - 2 * nt) / static_cast<int>(A_COLS);
+}
+constexpr int CONV_SETS = 3;               // sets of four converter warps, taking stages in turn
+constexpr int CONV_WARPS = 4 * CONV_SETS;  // converter warps 6..17 (quantised heads)
 constexpr int RAW_PRODUCER = 2 + EPI_WARPS + CONV_WARPS;  // warp streaming the quantised codes
 
 // Epilogue warps: W8A8's MMAs take half the time of bf16's per tile, so two
@@ -162,7 +179,7 @@ __host__ __device__ constexpr uint32_t raw_bytes() {
 // operand stages per raw stage (a raw stage holds 256 NVFP4 or 128 E4M3 columns)
 template <int HF>
 __host__ __device__ constexpr int raw_k() {
-  return (HF == HF_NVFP4 ? 256 : 128) / stage_k<HF>();
+  return (HF == HF_NVFP4 ? 256 : 128) / STAGE_K;
 }
 
 struct PairCtl {
@@ -212,27 +229,24 @@ __host__ __device__ constexpr size_t stage_area() {
 
 // Stage layout for a token group of NT rows (NT/2 in each CTA), one block per
 // atom: [A block 0 (| A block 1) | B block 0 (| B block 1)], A = 128 head
-// rows, B = NT/2 token rows (all NT for heads decoded in the kernel), each
+// rows (none for heads decoded in the kernel), B = NT/2 token rows, each
 // block 1 KB aligned.
 template <int HF>
 __host__ __device__ constexpr uint32_t stage_bytes(int nt) {
-  // heads decoded in the kernel: one CTA multiplies its 128 head rows by all NT token rows
-  return is_quant<HF>() ? A_BLOCK + static_cast<uint32_t>(nt) * ATOM_ROWS_BYTES
-                        : (stage_k<HF>() / atom_cols<HF>()) *
-                              (A_BLOCK + b_terms<HF>() * static_cast<uint32_t>(nt / 2) * ATOM_ROWS_BYTES);
+  return (STAGE_K / atom_cols<HF>()) * ((is_quant<HF>() ? 0u : A_BLOCK) +
+                                        b_terms<HF>() * static_cast<uint32_t>(nt / 2) * ATOM_ROWS_BYTES);
 }
-// Operand stages: as many as fit (at most MAX_STAGES) for bf16 heads; for
-// quantised heads at most QUANT_STAGES next to a raw ring of at least three
-// stages, which takes the rest of the area.
+// Operand stages: as many as fit, at most MAX_STAGES; for quantised heads next
+// to a raw ring of at least MIN_RAW stages, which takes the rest of the area,
+// no more than the A stages in tensor memory, and at most QUANT_STAGES.
 template <int HF, bool VERIFY>
 __host__ __device__ constexpr int stage_count(int nt) {
-  return is_quant<HF>()
-             ? (static_cast<int>((stage_area<HF, VERIFY>() - 3 * raw_bytes<HF>()) / stage_bytes<HF>(nt)) < QUANT_STAGES
-                    ? static_cast<int>((stage_area<HF, VERIFY>() - 3 * raw_bytes<HF>()) / stage_bytes<HF>(nt))
-                    : QUANT_STAGES)
-         : static_cast<int>(stage_area<HF, VERIFY>() / stage_bytes<HF>(nt)) < MAX_STAGES
-             ? static_cast<int>(stage_area<HF, VERIFY>() / stage_bytes<HF>(nt))
-             : MAX_STAGES;
+  int n = static_cast<int>((stage_area<HF, VERIFY>() - (is_quant<HF>() ? MIN_RAW * raw_bytes<HF>() : 0)) /
+                           stage_bytes<HF>(nt));
+  if (n > MAX_STAGES) n = MAX_STAGES;
+  if (is_quant<HF>() && n > a_stages(nt)) n = a_stages(nt);
+  if (is_quant<HF>() && n > QUANT_STAGES) n = QUANT_STAGES;
+  return n;
 }
 template <int HF, bool VERIFY>
 __host__ __device__ constexpr int raw_count(int nt) {
@@ -251,78 +265,64 @@ static_assert(stage_count<HF_E4M3X2, false>(160) == 5 && stage_count<HF_E4M3X2, 
               "two-term rows: five 36 KB stages at NT = 160, four 48 KB stages at NT = 256");
 static_assert(stage_count<HF_E4M3X2, true>(160) == 5 && stage_count<HF_E4M3X2, true>(256) == 4,
               "two-term rows: the same stages on the verification path");
-static_assert(stage_count<HF_NVFP4, false>(160) == 4 && stage_count<HF_E4M3, false>(160) == 4 &&
-                  stage_count<HF_NVFP4, true>(160) == 4 && stage_count<HF_E4M3, true>(160) == 4,
-              "four operand stages at NT = 160 for quantised heads");
-static_assert(stage_count<HF_NVFP4, true>(256) >= 3 && stage_count<HF_E4M3, true>(256) >= 3 &&
-                  raw_count<HF_NVFP4, true>(256) >= 3 && raw_count<HF_E4M3, true>(256) >= 3,
-              "three operand and three raw stages at NT = 256");
+// Sets of converter warps that take operand stages in turn. A barrier's parity
+// tells two neighbouring uses of a stage apart, so a set that comes to stage g
+// must know that use g - 2 NS of that operand stage is over, and that the raw
+// stage's last but one load was. It has finished stage g - sets, so all stages
+// up to g - sets - NS are multiplied: that takes sets <= NS, and (as a raw
+// stage may hold as little as one operand stage, where a tile ends) a raw ring
+// of at least sets + NS.
+__host__ __device__ constexpr int conv_sets(int stages) { return CONV_SETS < stages ? CONV_SETS : stages; }
+template <int HF, bool VERIFY>
+constexpr bool turns_ok(int nt) {
+  return stage_count<HF, VERIFY>(nt) >= 2 &&
+         raw_count<HF, VERIFY>(nt) >= conv_sets(stage_count<HF, VERIFY>(nt)) + stage_count<HF, VERIFY>(nt) &&
+         (nt <= 32 || turns_ok<HF, VERIFY>(nt - 32));
+}
+static_assert(turns_ok<HF_NVFP4, false>(QUANT_GROUP) && turns_ok<HF_NVFP4, true>(QUANT_GROUP) &&
+                  turns_ok<HF_E4M3, false>(QUANT_GROUP) && turns_ok<HF_E4M3, true>(QUANT_GROUP),
+              "converter sets in turn at every group size");
+static_assert(stage_count<HF_NVFP4, true>(QUANT_GROUP) == 2 && stage_count<HF_NVFP4, true>(160) == 3 &&
+                  stage_count<HF_NVFP4, true>(128) == 4,
+              "quantised heads: operand stages beside two accumulators");
 
-// Decodes this thread's share of one operand stage (128 head rows x 64
-// columns, global columns kcol0..) from the raw stage at raw_base into the
-// f16 (F16) or bf16 A tile at a_base (one SW128 atom); both are exact. h:
-// which 64-column part of the raw stage. Columns at or past d decode to zero.
-// ct: 0..CONV_THREADS-1.
+// Decodes 64 columns (global columns kcol0..) of one head row from the raw
+// stage at raw_base into f16 (F16) or bf16 pairs, the lower column in the low
+// half; both are exact. h: which 64-column part of the raw stage. Columns at or
+// past d decode to zero.
 template <int HF, bool F16>
-__device__ __forceinline__ void convert_stage(uint32_t raw_base, int h, uint32_t a_base, int ct, int kcol0, int d) {
-  static_assert(!is_quant<HF>() || stage_k<HF>() == 64, "one atom per quantised operand stage");
+__device__ __forceinline__ void decode_row(uint32_t raw_base, int h, int row, int kcol0, int d, uint32_t (&w)[32]) {
+  const uint32_t rowbase = raw_base + row * 128;
   if constexpr (HF == HF_NVFP4) {
+    const uint4 q0 = ld_shared_v4(rowbase + (((2 * h) ^ (row & 7)) << 4));
+    const uint4 q1 = ld_shared_v4(rowbase + (((2 * h + 1) ^ (row & 7)) << 4));
+    const uint32_t bs = ld_shared_u32(raw_base + RAW_CODE_BYTES + row * 16 + 4 * h);
+    const uint32_t s01 = e4m3x2_to_f16x2(bs & 0xFFFFu), s23 = e4m3x2_to_f16x2(bs >> 16);
+    const uint32_t sc[4] = {__byte_perm(s01, 0, 0x1010), __byte_perm(s01, 0, 0x3232), __byte_perm(s23, 0, 0x1010),
+                            __byte_perm(s23, 0, 0x3232)};
+    const uint32_t words[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
 #pragma unroll
-    for (int i = 0; i < 256 / CONV_THREADS; ++i) {
-      const int ci = ct + CONV_THREADS * i;
-      const int row = ci >> 1, j = ci & 1;  // 32-column chunk j of the stage
-      const int c = h * 2 + j;              // its 16 bytes of codes within the raw row
-      const uint4 q = ld_shared_v4(raw_base + row * 128 + ((c ^ (row & 7)) << 4));
-      const uint32_t s01 = e4m3x2_to_f16x2(ld_shared_u16(raw_base + RAW_CODE_BYTES + row * 16 + c * 2));
-      const uint32_t sc[2] = {__byte_perm(s01, 0, 0x1010), __byte_perm(s01, 0, 0x3232)};
-      const uint32_t words[4] = {q.x, q.y, q.z, q.w};
-      uint32_t w[16];
-#pragma unroll
-      for (int b = 0; b < 16; ++b)  // byte b: elements 2b (low nibble), 2b + 1; 16 elements per block scale
-      {
-        const uint32_t hv = hmul2_u32(e2m1x2_to_f16x2(__byte_perm(words[b >> 2], 0, 0x4440 + (b & 3))), sc[b >> 3]);
-        w[b] = F16 ? hv : f16x2_to_bf16x2(hv);
-      }
-      const int col0 = kcol0 + j * 32;
-      if (col0 + 32 > d) {
-#pragma unroll
-        for (int b = 0; b < 16; ++b) {
-          if (col0 + 2 * b >= d) w[b] = 0u;
-          else if (col0 + 2 * b + 1 >= d) w[b] &= 0xFFFFu;
-        }
-      }
-      const uint32_t rowbase = a_base + row * 128;
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        st_shared_v4(rowbase + (((j * 4 + u) ^ (row & 7)) << 4), w[4 * u], w[4 * u + 1], w[4 * u + 2], w[4 * u + 3]);
-    }
+    for (int b = 0; b < 32; ++b)  // byte b: elements 2b (low nibble), 2b + 1; 16 elements per block scale
+      w[b] = hmul2_u32(e2m1x2_to_f16x2(__byte_perm(words[b >> 2], 0, 0x4440 + (b & 3))), sc[b >> 3]);
   } else {
 #pragma unroll
-    for (int i = 0; i < 512 / CONV_THREADS; ++i) {
-      const int ci = ct + CONV_THREADS * i;
-      const int row = ci >> 2, j = ci & 3;  // 16-column chunk j of the stage
-      const int c = h * 4 + j;              // its 16 bytes of codes within the raw row
-      const uint4 q = ld_shared_v4(raw_base + row * 128 + ((c ^ (row & 7)) << 4));
+    for (int c = 0; c < 4; ++c) {
+      const uint4 q = ld_shared_v4(rowbase + (((4 * h + c) ^ (row & 7)) << 4));
       const uint32_t words[4] = {q.x, q.y, q.z, q.w};
-      uint32_t w[8];
 #pragma unroll
       for (int b = 0; b < 8; ++b)  // bytes 2b, 2b + 1: elements 2b, 2b + 1
-      {
-        const uint32_t hv = e4m3x2_to_f16x2(__byte_perm(words[b >> 1], 0, (b & 1) ? 0x4432 : 0x4410));
-        w[b] = F16 ? hv : f16x2_to_bf16x2(hv);
-      }
-      const int col0 = kcol0 + j * 16;
-      if (col0 + 16 > d) {
+        w[8 * c + b] = e4m3x2_to_f16x2(__byte_perm(words[b >> 1], 0, (b & 1) ? 0x4432 : 0x4410));
+    }
+  }
+  if constexpr (!F16) {
 #pragma unroll
-        for (int b = 0; b < 8; ++b) {
-          if (col0 + 2 * b >= d) w[b] = 0u;
-          else if (col0 + 2 * b + 1 >= d) w[b] &= 0xFFFFu;
-        }
-      }
-      const uint32_t rowbase = a_base + row * 128;
+    for (int b = 0; b < 32; ++b) w[b] = f16x2_to_bf16x2(w[b]);
+  }
+  if (kcol0 + 64 > d) {
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
-        st_shared_v4(rowbase + (((j * 2 + u) ^ (row & 7)) << 4), w[4 * u], w[4 * u + 1], w[4 * u + 2], w[4 * u + 3]);
+    for (int b = 0; b < 32; ++b) {
+      if (kcol0 + 2 * b >= d) w[b] = 0u;
+      else if (kcol0 + 2 * b + 1 >= d) w[b] &= 0xFFFFu;
     }
   }
 }
@@ -335,6 +335,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
                        const __grid_constant__ PairQuantMaps tmQ, const __grid_constant__ PairTokenMaps tmL,
                        TcArgs a) {
   constexpr bool QUANT = is_quant<HF>();
+  constexpr int MAX_CHUNKS = max_chunks<HF>();
   constexpr bool W8A8 = HF == HF_W8A8;
   constexpr bool X2 = HF == HF_E4M3X2;
   static_assert(!(W8A8 && VERIFY), "W8A8 serves the commit step");
@@ -350,28 +351,23 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   PairCtl* ctl = &tail->ctl;
   const uint32_t smem_base = smem_u32(smem);
 
-  // pairs per cluster: two sharing head tiles (mc = 2) or token rows (vc = 2);
-  // quantised heads run without clusters
-  const int MC = QUANT ? 1 : plan_mc(a.plan) * plan_vc(a.plan);
-  if constexpr (pair_cluster<HF>()) {
-    // launched without its cluster there is no peer CTA to map or to pair
-    // MMAs with: report and do nothing
-    if (cluster_nctarank() != static_cast<uint32_t>(2 * MC)) {
-      if (threadIdx.x == 0) atomicOr(a.status, DEV_BAD_LAUNCH);
-      return;
-    }
+  // pairs per cluster: two sharing head tiles (mc = 2) or token rows (vc = 2)
+  const int MC = plan_mc(a.plan) * plan_vc(a.plan);
+  // launched without its cluster there is no peer CTA to map or to pair
+  // MMAs with: report and do nothing
+  if (cluster_nctarank() != static_cast<uint32_t>(2 * MC)) {
+    if (threadIdx.x == 0) atomicOr(a.status, DEV_BAD_LAUNCH);
+    return;
   }
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const uint32_t crank = QUANT ? 0u : cluster_ctarank();
-  // 0: the CTA that issues the pair's MMAs (bf16 heads); quantised heads: the
-  // half of the v-tile this CTA takes on its own
-  const uint32_t rank = QUANT ? (blockIdx.x & 1u) : (crank & 1u);
+  const uint32_t crank = cluster_ctarank();
+  const uint32_t rank = crank & 1u;  // 0: the CTA that issues the pair's MMAs
   const int pp = static_cast<int>(crank >> 1);  // this pair's token group (vc = 1) or v-tile (vc = 2) in the runner
   const uint32_t lead = crank & ~1u;            // cluster rank of this pair's issuing CTA
   const uint32_t pair_mask = 3u << (2 * pp);    // both CTAs of this pair
   const uint32_t all_mask = (1u << (2 * MC)) - 1u;
-  const int pair = QUANT ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x) / (2 * MC);
+  const int pair = static_cast<int>(blockIdx.x) / (2 * MC);
 
   if (threadIdx.x == 0) {
     if constexpr (QUANT) {
@@ -379,20 +375,20 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
       if constexpr (HF == HF_NVFP4) prefetch_tmap(&tmQ.scales);
       for (int r = 0; r < MAX_RAW; ++r) {
         mbar_init(smem_u32(&ctl->rfull[r]), 1);
-        mbar_init(smem_u32(&ctl->rempty[r]), CONV_WARPS);
+        mbar_init(smem_u32(&ctl->rempty[r]), 4 * raw_k<HF>());  // a set of converter warps per operand stage
       }
     } else {
       prefetch_tmap(&tmW);
     }
     for (int s = 0; s < MAX_STAGES; ++s) {
-      // quantised heads: the token bytes' arrival plus the CTA's converter warps
-      mbar_init(smem_u32(&ctl->full[s]), QUANT ? 1 + CONV_WARPS : 1);
+      // the operand bytes' arrival; quantised heads: and a set of converter warps of each CTA
+      mbar_init(smem_u32(&ctl->full[s]), QUANT ? 1 + 2 * 4 : 1);
       // commits of the issuing CTA of every pair that reads this stage
       mbar_init(smem_u32(&ctl->empty[s]), static_cast<uint32_t>(MC));
     }
     for (int i = 0; i < MAX_ACC; ++i) {
       mbar_init(smem_u32(&ctl->tfull[i]), 1);
-      mbar_init(smem_u32(&ctl->tempty[i]), QUANT ? EW : 2 * EW);
+      mbar_init(smem_u32(&ctl->tempty[i]), 2 * EW);
     }
     mbar_init(smem_u32(&ctl->drain), 1);
     mbar_init(smem_u32(&ctl->epi_sync), EW * 32);
@@ -400,19 +396,11 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     fence_mbar_init();
   }
   if (warp == 1) {
-    if constexpr (QUANT) {
-      tmem_alloc(smem_u32(&ctl->tmem_base), TMEM_COLS);
-      tmem_relinquish();
-    } else {
-      tmem_alloc_pair(smem_u32(&ctl->tmem_base), TMEM_COLS);
-      tmem_relinquish_pair();
-    }
+    tmem_alloc_pair(smem_u32(&ctl->tmem_base), TMEM_COLS);
+    tmem_relinquish_pair();
   }
   tc_fence_before();
-  if constexpr (QUANT)
-    __syncthreads();
-  else
-    cluster_sync_all();  // barriers initialised and TMEM allocated in both CTAs
+  cluster_sync_all();  // barriers initialised and TMEM allocated in both CTAs
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   volatile int* abort_flag = &ctl->abort_flag;
@@ -425,26 +413,26 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   if (!spill) griddep_wait();
   if (!spill && a.plan.G2 > 0) griddep_launch_dependents();
   const int n_rows = hdr_word(a.n_rows, HDR_N);
-  const int VC = QUANT ? 1 : plan_vc(plan_resolve(a.plan, n_rows));
+  const int VC = plan_vc(plan_resolve(a.plan, n_rows));
   const int pp_mt = VC == 1 ? pp : 0;  // this pair's token group within the runner's m-tiles
-  constexpr int BK = stage_k<HF>();
+  constexpr int BK = STAGE_K;
   constexpr int ACOLS = atom_cols<HF>();
   constexpr int NATOM = BK / ACOLS;
   const int nk = cdiv(a.d, BK);
-  const int NT = pair_group_rows(n_rows);
+  const int NT = plan_bm(a.plan, n_rows);
   const int half = NT / 2;
   // accumulators in TMEM: three of 160 columns when a group has at most 160
-  // tokens (the epilogue of one tile then overlaps two tiles of MMAs), else two of 256
-  const uint32_t NACC = NT <= 160 ? 3u : 2u;
-  const uint32_t ACC_COLS = NT <= 160 ? 160u : 256u;
+  // tokens (the epilogue of one tile then overlaps two tiles of MMAs), else two
+  // of 256; quantised heads: two of NT below the A stages
+  const uint32_t NACC = !QUANT && NT <= 160 ? 3u : 2u;
+  const uint32_t ACC_COLS = QUANT ? static_cast<uint32_t>(NT) : NT <= 160 ? 160u : 256u;
+  const uint32_t A_TMEM = 2u * static_cast<uint32_t>(NT);
   const int nch = NT / 32;
   const uint32_t SB = stage_bytes<HF>(NT);
   const uint32_t B_BLOCK = static_cast<uint32_t>(half) * ATOM_ROWS_BYTES;
   const int STAGES = stage_count<HF, VERIFY>(NT);
   const int RSTAGES = raw_count<HF, VERIFY>(NT);
-  // bf16 heads: both CTAs' bytes land on the even CTA's barrier; quantised
-  // heads: this CTA's token rows only
-  const uint32_t tx_total = QUANT ? static_cast<uint32_t>(NT) * ATOM_ROWS_BYTES : 2u * SB;
+  const uint32_t tx_total = 2u * SB;  // both CTAs' bytes land on the even CTA's barrier
   const uint32_t raw_base = smem_base + static_cast<uint32_t>(STAGES) * SB;  // quantised heads' raw ring
   const CUtensorMap* tm_tok = &tmH.m[half / 8 - 1];  // box of exactly `half` rows
   const CUtensorMap* tm_lo = &tmL.m[half / 8 - 1];   // two-term rows: the lo terms
@@ -468,7 +456,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     it.init(a.plan, a.n_rows, pair);
     bool ok = true;
     while (ok && it.next_unit()) {
-      const int tok0 = (it.m_tile + pp_mt) * NT + (QUANT ? 0 : static_cast<int>(rank) * half);
+      const int tok0 = (it.m_tile + pp_mt) * NT + static_cast<int>(rank) * half;
       for (int step = it.vt; ok && step < it.vt_end; ++step) {
         int vt = step * VC + (VC == 2 ? pp : 0);
         // vc = 2 and an odd v-tile count: the last step's second v-tile lies past
@@ -482,15 +470,13 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
           }
           if (leader) {
             const uint32_t sa = smem_base + stage * SB;
+            if (rank == 0) mbar_expect_tx(smem_u32(&ctl->full[stage]), tx_total);
+            const uint32_t fb = full0_leader + 8u * stage;
             if constexpr (QUANT) {
-              // all NT token rows of the group, as two boxes of NT/2 rows
-              const uint32_t fb = smem_u32(&ctl->full[stage]);
-              mbar_expect_tx(fb, tx_total);
-              tma_load_2d(sa + A_BLOCK, tm_tok, fb, kb * BK, tok0, pol_h);
-              tma_load_2d(sa + A_BLOCK + B_BLOCK, tm_tok, fb, kb * BK, tok0 + half, pol_h);
+#pragma unroll
+              for (int j = 0; j < NATOM; ++j)
+                tma_load_2d_pair(sa + j * B_BLOCK, tm_tok, fb, kb * BK + ACOLS * j, tok0, pol_h);
             } else {
-              if (rank == 0) mbar_expect_tx(smem_u32(&ctl->full[stage]), tx_total);
-              const uint32_t fb = full0_leader + 8u * stage;
 #pragma unroll
               for (int j = 0; j < NATOM; ++j) {
                 // the head atom's 128 rows as two boxes of 64: both loaded here, or
@@ -536,12 +522,12 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
         if (issued_mask & (1u << s)) mbar_drain(smem_u32(&ctl->full[s]), (issued_phase >> s) & 1u);
     __syncwarp();
   } else if (warp == 1) {
-    // ------------------------------------------------------ MMA issuer (even CTA; every CTA for quantised heads)
-    if (rank == 0 || QUANT) {
+    // ------------------------------------------------------ MMA issuer (even CTA)
+    if (rank == 0) {
       const bool leader = elect_one();
       const uint32_t idesc = (W8A8 || X2) ? idesc_e4m3_f32(256, NT)
-                             : F16OPS ? idesc_f16_f32(128, NT)
-                                      : idesc_bf16_f32(QUANT ? 128 : 256, NT);
+                             : F16OPS ? idesc_f16_f32(256, NT)
+                                      : idesc_bf16_f32(256, NT);
       uint32_t stage = 0, phase = 0;
       uint32_t acc = 0, acc_phase = 0;
       TileIter it;
@@ -563,15 +549,17 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
             tc_fence_after();
             if (leader) {
               const uint32_t sa = smem_base + stage * SB;
+              const uint32_t a_tmem = tmem_base + A_TMEM + stage * A_COLS;
 #pragma unroll
               for (int j = 0; j < NATOM; ++j) {
                 const uint64_t adesc = sw128_kmajor_desc(sa + j * A_BLOCK);
-                const uint64_t bdesc = sw128_kmajor_desc(sa + NATOM * A_BLOCK + j * B_BLOCK);
+                const uint64_t bdesc = sw128_kmajor_desc(sa + (QUANT ? 0 : NATOM * A_BLOCK) + j * B_BLOCK);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                   // +32 bytes along K per MMA (16 bf16 / 32 E4M3 columns) = +2 in the address field
                   if constexpr (QUANT) {
-                    umma_bf16(d_tmem, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | j | k) != 0);
+                    // 16 elements of A per MMA: 8 columns of tensor memory
+                    umma_f16_pair_ta(d_tmem, a_tmem + 32u * j + 8u * k, bdesc + 2u * k, idesc, (kb | j | k) != 0);
                   } else if constexpr (X2) {
                     // the head atom times the hi terms, then times the lo terms
                     const uint64_t ldesc = sw128_kmajor_desc(sa + A_BLOCK + B_BLOCK);
@@ -584,10 +572,8 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
                   }
                 }
               }
-              if constexpr (QUANT)
-                umma_commit(smem_u32(&ctl->empty[stage]));
-              else  // the stage's head halves came from both pairs: free it in every CTA
-                umma_commit_pair_mc(smem_u32(&ctl->empty[stage]), static_cast<uint16_t>(all_mask));
+              // the stage's head halves came from both pairs: free it in every CTA
+              umma_commit_pair_mc(smem_u32(&ctl->empty[stage]), static_cast<uint16_t>(all_mask));
             }
             __syncwarp();
             if (++stage == STAGES) {
@@ -596,12 +582,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
             }
           }
           if (!ok) break;
-          if (leader) {
-            if constexpr (QUANT)
-              umma_commit(smem_u32(&ctl->tfull[acc]));
-            else
-              umma_commit_pair_mc(smem_u32(&ctl->tfull[acc]), static_cast<uint16_t>(pair_mask));
-          }
+          if (leader) umma_commit_pair_mc(smem_u32(&ctl->tfull[acc]), static_cast<uint16_t>(pair_mask));
           __syncwarp();
           if (++acc == NACC) {
             acc = 0;
@@ -610,10 +591,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
         }
       }
       if (leader) {
-        if constexpr (QUANT)
-          umma_commit(smem_u32(&ctl->drain));
-        else
-          umma_commit_pair_mc(smem_u32(&ctl->drain), static_cast<uint16_t>(1u << crank));
+        umma_commit_pair_mc(smem_u32(&ctl->drain), static_cast<uint16_t>(1u << crank));
         mbar_drain(smem_u32(&ctl->drain), 0);
       }
       __syncwarp();
@@ -660,39 +638,68 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     __syncwarp();
   } else if (QUANT && warp >= 2 + EPI_WARPS) {
     // ------------------------------------------------------ converters (quantised heads)
-    const int ct = threadIdx.x - (2 + EPI_WARPS) * 32;  // 0..CONV_THREADS-1
-    const int RS = RSTAGES;
+    const int set = (warp - 2 - EPI_WARPS) / 4;
+    const int quarter = warp & 3;  // the tensor-memory lanes this warp may write
+    const int row = quarter * 32 + lane;
+    const uint32_t a_lane = tmem_base + A_TMEM + (static_cast<uint32_t>(quarter * 32) << 16);
+    const uint32_t full_leader0 = mapa_shared(smem_u32(&ctl->full[0]), lead);
+    const uint32_t RS = static_cast<uint32_t>(RSTAGES), NS = static_cast<uint32_t>(STAGES);
     constexpr int RK = raw_k<HF>();
-    uint32_t r = 0, rph = 0, stage = 0, phase = 0;
+    uint32_t r = 0, rph = 0, st = 0, ph = 0;  // raw and operand stage of the current columns, with their phases
+    const int sets = conv_sets(STAGES);
+    int turn = 0;  // the set that takes the current operand stage
     TileIter it;
     it.init(a.plan, a.n_rows, pair);
     bool ok = true;
     while (ok && it.next_unit()) {
       for (int vt = it.vt; ok && vt < it.vt_end; ++vt) {
         for (int kb = 0; kb < nk; ++kb) {
-          const int h = kb % RK;
-          if (h == 0 && !mbar_wait_warp(smem_u32(&ctl->rfull[r]), rph, abort_flag, a.status)) {
-            ok = false;
-            break;
-          }
-          if (!mbar_wait_warp(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag, a.status)) {
-            ok = false;
-            break;
-          }
-          convert_stage<HF, F16OPS>(raw_base + r * raw_bytes<HF>(), h, smem_base + stage * SB, ct, kb * BK, a.d);
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&ctl->full[stage]));
-          if (h == RK - 1 || kb == nk - 1) {
-            if (lane == 0) mbar_arrive(smem_u32(&ctl->rempty[r]));
-            if (++r == static_cast<uint32_t>(RS)) {
-              r = 0;
-              rph ^= 1u;
+          const int h = kb % RK;                           // this operand stage's place in the raw stage
+          const bool last = h == RK - 1 || kb == nk - 1;  // the raw stage's last operand stage
+          if (turn == set) {
+            // asked before the decode, so that a free stage costs no wait after it
+            const uint32_t is_free = mbar_test_wait(smem_u32(&ctl->empty[st]), ph ^ 1u);
+            if (!mbar_wait_warp(smem_u32(&ctl->rfull[r]), rph, abort_flag, a.status)) {
+              ok = false;
+              break;
+            }
+#pragma unroll
+            for (int p = 0; p < PARTS; ++p) {
+              uint32_t w[32];
+              decode_row<HF, F16OPS>(raw_base + r * raw_bytes<HF>(), h * PARTS + p, row, kb * BK + p * PART_K, a.d, w);
+              if (p == 0) {
+                if (!__all_sync(0xffffffffu, is_free) &&
+                    !mbar_wait_warp(smem_u32(&ctl->empty[st]), ph ^ 1u, abort_flag, a.status)) {
+                  ok = false;
+                  break;
+                }
+                tc_fence_after();
+              }
+              tmem_st32(a_lane + st * A_COLS + 32u * p, w);
+            }
+            if (!ok) break;
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+              if (rank == 0)
+                mbar_arrive(smem_u32(&ctl->full[st]));
+              else
+                mbar_arrive_cluster_relaxed(full_leader0 + 8u * st);
+              mbar_arrive(smem_u32(&ctl->rempty[r]));
+              // a raw stage the tile ends in counts its missing operand stages here
+              if (last)
+                for (int q = h + 1; q < RK; ++q) mbar_arrive(smem_u32(&ctl->rempty[r]));
             }
           }
-          if (++stage == static_cast<uint32_t>(STAGES)) {
-            stage = 0;
-            phase ^= 1u;
+          turn = turn + 1 == sets ? 0 : turn + 1;
+          if (++st == NS) {
+            st = 0;
+            ph ^= 1u;
+          }
+          if (last && ++r == RS) {
+            r = 0;
+            rph ^= 1u;
           }
         }
       }
@@ -847,10 +854,10 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          if (rank == 0 || QUANT)
+          if (rank == 0)
             mbar_arrive(tempty_local0 + 8u * acc);
           else
-            mbar_arrive_cluster(tempty_leader0 + 8u * acc);
+            mbar_arrive_cluster_relaxed(tempty_leader0 + 8u * acc);
         }
         if (++acc == NACC) {
           acc = 0;
@@ -918,17 +925,9 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   __syncwarp();
   griddep_launch_dependents();
   tc_fence_before();
-  if constexpr (QUANT)
-    __syncthreads();
-  else
-    cluster_sync_all();  // both CTAs done: no MMA, copy or remote arrival is pending
+  cluster_sync_all();  // both CTAs done: no MMA, copy or remote arrival is pending
   tc_fence_after();
-  if (warp == 1) {
-    if constexpr (QUANT)
-      tmem_dealloc(tmem_base, TMEM_COLS);
-    else
-      tmem_dealloc_pair(tmem_base, TMEM_COLS);
-  }
+  if (warp == 1) tmem_dealloc_pair(tmem_base, TMEM_COLS);
   // the spill launch completes only after the main launch: the kernel after
   // it (the merge) waits on this grid alone
   if (spill) griddep_wait();
@@ -952,9 +951,9 @@ static cudaError_t pair_opt_in() {
   return cudaSuccess;
 }
 
-// runners: clusters of `mc` CTA pairs (mc = 1 without clusters for quantised heads)
+// runners: clusters of `mc` CTA pairs
 static void pair_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int runners, int threads, cudaStream_t st,
-                        bool programmatic, bool cluster = true, int mc = 1) {
+                        bool programmatic, int mc) {
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3(2 * mc * runners, 1, 1);
   cfg->blockDim = dim3(threads, 1, 1);
@@ -962,13 +961,11 @@ static void pair_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int 
   cfg->stream = st;
   cfg->attrs = attr;
   cfg->numAttrs = 0;
-  if (cluster) {
-    attr[cfg->numAttrs].id = cudaLaunchAttributeClusterDimension;
-    attr[cfg->numAttrs].val.clusterDim.x = 2 * mc;
-    attr[cfg->numAttrs].val.clusterDim.y = 1;
-    attr[cfg->numAttrs].val.clusterDim.z = 1;
-    ++cfg->numAttrs;
-  }
+  attr[cfg->numAttrs].id = cudaLaunchAttributeClusterDimension;
+  attr[cfg->numAttrs].val.clusterDim.x = 2 * mc;
+  attr[cfg->numAttrs].val.clusterDim.y = 1;
+  attr[cfg->numAttrs].val.clusterDim.z = 1;
+  ++cfg->numAttrs;
   if (programmatic) {
     attr[cfg->numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[cfg->numAttrs].val.programmaticStreamSerializationAllowed = 1;
@@ -981,7 +978,7 @@ cudaError_t lmhead_pair_max_clusters(int sm_count, int mc, int* clusters) {
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  pair_config(&cfg, attr, sm_count / (2 * mc), pair_threads<HF_BF16>(), nullptr, false, true, mc);
+  pair_config(&cfg, attr, sm_count / (2 * mc), pair_threads<HF_BF16>(), nullptr, false, mc);
   int n = 0;
   e = cudaOccupancyMaxActiveClusters(&n, lmhead_pair_kernel<HF_BF16, false>, &cfg);
   if (e != cudaSuccess) return e;
@@ -1000,10 +997,10 @@ static cudaError_t launch_pair(const PairTokenMaps& tmH, const CUtensorMap& tmW,
   if (a.plan.G2 > 0) {
     // clusters of two pairs and the spill launch of single pairs behind them
     // (the header's vocabulary split assumes both run)
-    if (!pair_cluster<HF>() || ppc != 2) return cudaErrorInvalidValue;
+    if (is_quant<HF>() || ppc != 2) return cudaErrorInvalidValue;
     TcArgs main = a;
     main.plan.role = 0;
-    pair_config(&cfg, attr, a.plan.G, pair_threads<HF>(), st, true, true, 2);
+    pair_config(&cfg, attr, a.plan.G, pair_threads<HF>(), st, true, 2);
     e = cudaLaunchKernelEx(&cfg, lmhead_pair_kernel<HF, VERIFY>, tmH, tmW, tmQ, tmL, main);
     if (e != cudaSuccess) return e;
     TcArgs side = a;
@@ -1012,11 +1009,11 @@ static cudaError_t launch_pair(const PairTokenMaps& tmH, const CUtensorMap& tmW,
     side.plan.mc = 1;
     side.plan.vc = 1;
     side.plan.cpu = SPILL_UNIT_SLOTS;
-    pair_config(&cfg, attr, side.plan.G, pair_threads<HF>(), st, true, true, 1);
+    pair_config(&cfg, attr, side.plan.G, pair_threads<HF>(), st, true, 1);
     return cudaLaunchKernelEx(&cfg, lmhead_pair_kernel<HF, VERIFY>, tmH, tmW, tmQ, tmL, side);
   }
-  if (!pair_cluster<HF>() && ppc != 1) return cudaErrorInvalidValue;
-  pair_config(&cfg, attr, a.plan.G, pair_threads<HF>(), st, true, pair_cluster<HF>(), pair_cluster<HF>() ? ppc : 1);
+  if (is_quant<HF>() && ppc != 1) return cudaErrorInvalidValue;
+  pair_config(&cfg, attr, a.plan.G, pair_threads<HF>(), st, true, ppc);
   return cudaLaunchKernelEx(&cfg, lmhead_pair_kernel<HF, VERIFY>, tmH, tmW, tmQ, tmL, a);
 }
 

@@ -1,5 +1,6 @@
 """Windows around one token group (256 compacted rows), where the clusters' layout is chosen on the device: the two
-pairs share token rows for a single group and head tiles for two. Every position is compared with a float64
+pairs share token rows for a single group and head tiles for two; and around the group sizes of heads decoded in the
+kernel (at most 192 rows, with four, three or two operand stages in flight). Every position is compared with a float64
 evaluation, over vocabularies of one, three (an odd last pair of v-tiles) and many v-tiles, and with workspaces that
 hold the partial slots of both layouts or only of the second.
 """
@@ -35,6 +36,17 @@ def make(head, P, V, d, seed):
     if head == "bf16":
         w = w.bfloat16()
         return h, w, None, h64 @ w.double().t()
+    if head == "nvfp4":
+        pad = (-((d + 15) // 16)) % 16  # 16-byte aligned rows of codes and block scales
+        codes = torch.randint(0, 256, (V, (d + 31) // 32 * 16), generator=g, device="cuda", dtype=torch.int32)
+        bs = torch.randint(40, 60, (V, (d + 15) // 16 + pad), generator=g, device="cuda", dtype=torch.int32)
+        scale = (torch.rand(V, generator=g, device="cuda") + 0.5) / d ** 0.5
+        nib = torch.stack([codes & 15, codes >> 4], 2).view(V, -1)[:, :d]
+        val = torch.tensor([0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 6.0], device="cuda")[(nib & 7).long()] * (1 - 2 * (nib >> 3))
+        bs = bs.to(torch.uint8)
+        block = bs.view(torch.float8_e4m3fn).double().repeat_interleave(16, 1)[:, :d]
+        w64 = val.double() * block * scale[:, None].double()
+        return h, bdc.Nvfp4Head(codes.to(torch.uint8), bs, d), scale, h64 @ w64.t()
     scale = w.abs().amax(1) / 448
     w = (w / scale[:, None]).to(torch.float8_e4m3fn)
     return h, w, scale, h64 @ (w.double() * scale[:, None].double()).t()
@@ -74,9 +86,25 @@ def test_commit_step(head, V, N, monkeypatch):
         assert torch.equal(tok[live][sure].long(), logit[live].argmax(1)[sure])
 
 
-@pytest.mark.parametrize("n_req", [1, 51, 52, 60])  # 5, 255, 260 and 300 rows
+@pytest.mark.parametrize("N", [1, 32, 33, 96, 97, 128, 129, 160, 161, 192, 193, 300, 385, 9001])
+@pytest.mark.parametrize("V,d", [(200, 336), (5001, 64), (19001, 640), (700, 1056)])
+@pytest.mark.parametrize("head", ["nvfp4", "e4m3"])
+def test_head_decoded_in_the_kernel(head, V, d, N, monkeypatch):
+    monkeypatch.setenv("BD_E4M3_SPLIT", "0")
+    h, w, scale, logit = make(head, N, V, d, N)
+    ones = torch.ones(N, dtype=torch.uint8, device="cuda")
+    tok, conf, _, _ = bdc.commit_step(h, w, ones, ones, N, 1, 1, [0.5], weight_scale=scale)
+    assert bdc.bd_get_device_status() == 0
+    top = logit.topk(2, dim=1).values
+    # as above, with logits of at most ~40 and 1056 products
+    assert float((conf.double() - (top[:, 0] - logit.logsumexp(1)).exp()).abs().max()) < 2e-3
+    sure = top[:, 0] - top[:, 1] > 4e-3
+    assert torch.equal(tok[sure].long(), logit.argmax(1)[sure])
+
+
+@pytest.mark.parametrize("n_req", [1, 38, 51, 52, 60])  # 5, 190, 255, 260 and 300 rows
 @pytest.mark.parametrize("V", [200, 700, 19001])
-@pytest.mark.parametrize("head", ["bf16", "e4m3"])
+@pytest.mark.parametrize("head", ["bf16", "e4m3", "nvfp4"])
 def test_verify_step(head, V, n_req):
     D, d, eps = 4, 336, [0.3, 0.05]
     R = n_req * (D + 1)
