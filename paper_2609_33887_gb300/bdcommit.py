@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from ctypes import POINTER, c_float, c_int, c_int32, c_int64, c_size_t, c_void_p
 from dataclasses import dataclass
 from typing import Optional, Sequence
@@ -167,10 +168,16 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
-def make_hidden(hidden: torch.Tensor) -> bd_hidden:
-    if hidden.dim() != 2 or hidden.stride(1) != 1:
+def _hidden_fields(hidden: torch.Tensor) -> tuple:
+    ld, inner = hidden.stride() if hidden.dim() == 2 else (0, 0)
+    if inner != 1:
         raise ValueError("hidden must be a 2-D tensor with contiguous rows")
-    return bd_hidden(_ptr(hidden), _DT[hidden.dtype], hidden.shape[0], hidden.shape[1], hidden.stride(0))
+    rows, cols = hidden.shape
+    return hidden.data_ptr(), _DT[hidden.dtype], rows, cols, ld
+
+
+def make_hidden(hidden: torch.Tensor) -> bd_hidden:
+    return bd_hidden(*_hidden_fields(hidden))
 
 
 @dataclass
@@ -184,26 +191,36 @@ class Nvfp4Head:
     dim: int
 
 
-def make_weight(weight, scale: Optional[torch.Tensor] = None) -> bd_weight:
+def _weight_fields(weight, scale: Optional[torch.Tensor] = None) -> tuple:
     if isinstance(weight, Nvfp4Head):
         c, b = weight.codes, weight.block_scale
         if c.dtype != torch.uint8 or b.dtype != torch.uint8 or c.dim() != 2 or b.dim() != 2 \
                 or c.stride(1) != 1 or b.stride(1) != 1:
             raise ValueError("NVFP4 codes and block scales must be 2-D uint8 tensors with contiguous rows")
-        return bd_weight(_ptr(c), BD_NVFP4, c.shape[0], weight.dim, c.stride(0), _ptr(scale), _ptr(b), b.stride(0))
-    if weight.dim() != 2 or weight.stride(1) != 1:
+        return (c.data_ptr(), BD_NVFP4, c.shape[0], weight.dim, c.stride(0), _ptr(scale), b.data_ptr(), b.stride(0))
+    ld, inner = weight.stride() if weight.dim() == 2 else (0, 0)
+    if inner != 1:
         raise ValueError("weight must be a 2-D [vocab, dim] tensor with contiguous rows")
-    return bd_weight(_ptr(weight), _DT[weight.dtype], weight.shape[0], weight.shape[1], weight.stride(0),
-                     _ptr(scale), None, 0)
+    vocab, dim = weight.shape
+    return weight.data_ptr(), _DT[weight.dtype], vocab, dim, ld, _ptr(scale), None, 0
 
 
-def make_mask_state(pos_masked: torch.Tensor, block_flags: torch.Tensor, n_seq: int, n_slots: int,
-                    block_len: int, mask_token_id: int = -1) -> bd_mask_state:
+def make_weight(weight, scale: Optional[torch.Tensor] = None) -> bd_weight:
+    return bd_weight(*_weight_fields(weight, scale))
+
+
+def _mask_state_fields(pos_masked: torch.Tensor, block_flags: torch.Tensor, n_seq: int, n_slots: int,
+                       block_len: int, mask_token_id: int = -1) -> tuple:
     if pos_masked.dtype != torch.uint8 or block_flags.dtype != torch.uint8:
         raise ValueError("pos_masked and block_flags must be uint8")
     if not (pos_masked.is_contiguous() and block_flags.is_contiguous()):
         raise ValueError("pos_masked and block_flags must be contiguous")
-    return bd_mask_state(n_seq, n_slots, block_len, mask_token_id, _ptr(pos_masked), _ptr(block_flags))
+    return n_seq, n_slots, block_len, mask_token_id, pos_masked.data_ptr(), block_flags.data_ptr()
+
+
+def make_mask_state(pos_masked: torch.Tensor, block_flags: torch.Tensor, n_seq: int, n_slots: int,
+                    block_len: int, mask_token_id: int = -1) -> bd_mask_state:
+    return bd_mask_state(*_mask_state_fields(pos_masked, block_flags, n_seq, n_slots, block_len, mask_token_id))
 
 
 def make_tau_grid(tau: Sequence[float]):
@@ -213,10 +230,62 @@ def make_tau_grid(tau: Sequence[float]):
 
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
+        if torch.cuda.is_initialized():  # the handle alone, without a Stream object around it
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+# The structures of one call packed into one buffer with a single format: a
+# ctypes object per structure and pointer costs more host time than the
+# library's own part of a step (a commit_step call 37 us of host time with them, 26 us without).
+class _StepArgs(ctypes.Structure):
+    _fields_ = [("h", bd_hidden), ("w", bd_weight), ("ms", bd_mask_state), ("grid", bd_tau_grid), ("ex", bd_exec),
+                ("values", c_float * 32)]
+
+
+class _VerifyArgs(ctypes.Structure):
+    _fields_ = [("h", bd_hidden), ("w", bd_weight), ("dr", bd_draft), ("grid", bd_eps_grid), ("ex", bd_exec),
+                ("values", c_float * 32)]
+
+
+_STEP = struct.Struct("PiqqqPiqqqPPqiiiiPPPiPPNPPPii")
+_VERIFY = struct.Struct("PiqqqPiqqqPPqiiPPiPPNPPPii")
+assert _STEP.size == _StepArgs.values.offset and _VERIFY.size == _VerifyArgs.values.offset
+_VALUES = [struct.Struct("%df" % n) for n in range(33)]
+_void_fns = {}  # the same entry points, taking addresses
+
+
+def _void_fn(name: str, nargs: int):
+    fn = _void_fns.get(name)
+    if fn is None:
+        address = ctypes.cast(getattr(load_library(), name), c_void_p).value
+        fn = _void_fns[name] = ctypes.CFUNCTYPE(c_int, *[c_void_p] * nargs)(address)
+    return fn
+
+
+def _pack(fmt, args_type, values, before, after):
+    """(buffer, its address): `before`, the grid of `values`, then `after`, as args_type lays
+    them out; None where a value does not fit the format (ctypes then converts it its own way)."""
+    n = len(values)
+    if n > 32:
+        return None
+    buf = bytearray(ctypes.sizeof(args_type))
+    base = ctypes.addressof(ctypes.c_char.from_buffer(buf))
+    try:
+        fmt.pack_into(buf, 0, *before, base + fmt.size, n, *after)
+        _VALUES[n].pack_into(buf, fmt.size, *values)
+    except (struct.error, OverflowError, TypeError):
+        return None
+    return buf, base
+
+
+def _exec_fields(stream, workspace, out_counts, lmhead_events, variant, flags) -> tuple:
+    ws, ws_bytes = (0, 0) if workspace is None else (workspace.data_ptr(), workspace.numel() * workspace.element_size())
+    begin, end = (0, 0) if lmhead_events is None else (lmhead_events[0].cuda_event, lmhead_events[1].cuda_event)
+    return _stream_handle(stream) or 0, ws, ws_bytes, _ptr(out_counts) or 0, begin or 0, end or 0, variant, flags
 
 
 # ------------------------------------------------------------ entry points --
@@ -292,21 +361,19 @@ def bd_commit_step_ex(hidden, weight, weight_scale, pos_masked, block_flags, n_s
 
     All tensors are device tensors; `tau` is a host sequence of floats.
     Returns the bd_status code (0 on success)."""
-    h = make_hidden(hidden)
-    w = make_weight(weight, weight_scale)
-    ms = make_mask_state(pos_masked, block_flags, n_seq, n_slots, block_len, mask_token_id)
+    hf = _hidden_fields(hidden)
+    wf = _weight_fields(weight, weight_scale)
+    mf = _mask_state_fields(pos_masked, block_flags, n_seq, n_slots, block_len, mask_token_id)
+    ef = _exec_fields(stream, workspace, out_counts, lmhead_events, variant, flags)
+    packed = _pack(_STEP, _StepArgs, tau, (*hf, *wf[:5], wf[5] or 0, wf[6] or 0, wf[7], *mf), ef)
+    if packed is not None:
+        A = _StepArgs
+        base = packed[1]
+        return _void_fn("bd_commit_step_ex", 8)(
+            base + A.h.offset, base + A.w.offset, base + A.ms.offset, base + A.grid.offset,
+            _ptr(out_tokens), _ptr(out_conf), _ptr(out_commit), base + A.ex.offset)
+    h, w, ms, ex = bd_hidden(*hf), bd_weight(*wf), bd_mask_state(*mf), bd_exec(*ef)
     tg, _keep = make_tau_grid(tau)
-    ex = bd_exec()
-    ex.stream = _stream_handle(stream)
-    if workspace is not None:
-        ex.workspace = workspace.data_ptr()
-        ex.workspace_bytes = workspace.numel() * workspace.element_size()
-    ex.out_counts = _ptr(out_counts)
-    if lmhead_events is not None:
-        ex.lmhead_event_begin = lmhead_events[0].cuda_event
-        ex.lmhead_event_end = lmhead_events[1].cuda_event
-    ex.variant = variant
-    ex.flags = flags
     return int(load_library().bd_commit_step_ex(
         ctypes.byref(h), ctypes.byref(w), ctypes.byref(ms), ctypes.byref(tg),
         _ptr(out_tokens), _ptr(out_conf), _ptr(out_commit), ctypes.byref(ex)))
@@ -496,18 +563,19 @@ def bd_verify_workspace_size(hidden, weight, weight_scale, draft, n_req, n_draft
 def bd_verify_step(hidden, weight, weight_scale, draft, n_req, n_draft, eps, out_tokens, out_p_draft, out_entropy,
                    out_accept, out_accepted, stream=None, workspace=None, lmhead_events=None, variant=0) -> int:
     """Speculative-decoding verification (include/bdcommit.h); returns the status."""
-    h, w = make_hidden(hidden), make_weight(weight, weight_scale)
+    hf, wf = _hidden_fields(hidden), _weight_fields(weight, weight_scale)
+    ef = _exec_fields(stream, workspace, None, lmhead_events, variant, 0)
+    packed = _pack(_VERIFY, _VerifyArgs, eps,
+                   (*hf, *wf[:5], wf[5] or 0, wf[6] or 0, wf[7], n_req, n_draft, _ptr(draft) or 0), ef)
+    if packed is not None:
+        A = _VerifyArgs
+        base = packed[1]
+        return _void_fn("bd_verify_step", 10)(
+            base + A.h.offset, base + A.w.offset, base + A.dr.offset, base + A.grid.offset, _ptr(out_tokens),
+            _ptr(out_p_draft), _ptr(out_entropy), _ptr(out_accept), _ptr(out_accepted), base + A.ex.offset)
+    h, w, ex = bd_hidden(*hf), bd_weight(*wf), bd_exec(*ef)
     dr = bd_draft(n_req, n_draft, _ptr(draft))
     eg, _keep = make_eps_grid(eps)
-    ex = bd_exec()
-    ex.stream = _stream_handle(stream)
-    if workspace is not None:
-        ex.workspace = workspace.data_ptr()
-        ex.workspace_bytes = workspace.numel() * workspace.element_size()
-    if lmhead_events is not None:
-        ex.lmhead_event_begin = lmhead_events[0].cuda_event
-        ex.lmhead_event_end = lmhead_events[1].cuda_event
-    ex.variant = variant
     return load_library().bd_verify_step(ctypes.byref(h), ctypes.byref(w), ctypes.byref(dr), ctypes.byref(eg),
                                          _ptr(out_tokens), _ptr(out_p_draft), _ptr(out_entropy), _ptr(out_accept),
                                          _ptr(out_accepted), ctypes.byref(ex))
