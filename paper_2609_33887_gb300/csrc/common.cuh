@@ -246,9 +246,22 @@ __host__ __device__ __forceinline__ void plan_gv_range(const BandPlan& p, int* l
   }
 }
 
+// The choice for a single runner m-tile: one band and one round whatever gv, so
+// the fewest parts that keep the longest part shortest.
+__host__ __device__ __forceinline__ bool plan_single(const BandPlan& p, int n_mt, int* gm_out, int* gv_out) {
+  if (n_mt > 1) return false;
+  int lo, hi;
+  plan_gv_range(p, &lo, &hi);
+  if (hi < 1) hi = 1;  // an empty range of v-tiles
+  *gm_out = 1;
+  *gv_out = lo == hi || p.n_vt < 1 ? hi : cdiv(p.n_vt, cdiv(p.n_vt, hi));
+  return true;
+}
+
 // (GM, gv) for n_mt runner m-tiles, sequentially (host).
 __host__ __device__ __forceinline__ void plan_choose(const BandPlan& p, int n_rows, int* gm_out, int* gv_out) {
   const int n_mt = plan_runner_mts(p, n_rows) > 0 ? plan_runner_mts(p, n_rows) : 1;
+  if (plan_single(p, n_mt, gm_out, gv_out)) return;
   int glo, ghi, vlo, vhi;
   plan_gm_range(p, plan_bm(p, n_rows), n_mt, &glo, &ghi);
   plan_gv_range(p, &vlo, &vhi);
@@ -272,9 +285,12 @@ __host__ __device__ __forceinline__ void plan_choose(const BandPlan& p, int n_ro
 }
 
 #ifdef __CUDACC__
-// One word per warp of the CTA that evaluates the plan.
+// Shared memory of the CTA that evaluates the plan: a word per warp, and the
+// first candidates' costs (saturated) for the second pass.
 struct PlanScratch {
+  static constexpr int KEPT = 2048;
   uint64_t w[32];
+  uint32_t cost[KEPT];
 };
 
 // The smallest v over the CTA's threads.
@@ -293,45 +309,34 @@ __device__ __forceinline__ uint64_t cta_min(uint64_t v, PlanScratch* sh) {
 
 // The same choice by a whole CTA, a candidate per thread (the kernel that
 // learns N calls it once and stores GM and gv in the workspace header). The
-// LM head waits for it: with 256 threads instead of one warp the 912
-// candidates of a 77-row float32 window take a few microseconds of what was a
-// 29.7 us kernel.
+// LM head waits for it, so the code stays short: with 256 threads instead of
+// one warp the 912 candidates of a 77-row float32 window took a few
+// microseconds of what was a 29.7 us kernel, and windows of one runner m-tile
+// (all on clusters up to 512 rows) need no search.
 __device__ __forceinline__ void plan_choose_cta(const BandPlan& p, int n_rows, int* gm_out, int* gv_out,
                                                 PlanScratch* sh) {
   const int n_mt = plan_runner_mts(p, n_rows) > 0 ? plan_runner_mts(p, n_rows) : 1;
+  if (plan_single(p, n_mt, gm_out, gv_out)) return;
   int glo, ghi, vlo, vhi;
   plan_gm_range(p, plan_bm(p, n_rows), n_mt, &glo, &ghi);
   plan_gv_range(p, &vlo, &vhi);
   const int nv = vhi - vlo + 1;
   const int total = (ghi - glo + 1) * nv;
   const int t = static_cast<int>(threadIdx.x), nt = static_cast<int>(blockDim.x);
-  // the first CACHED candidates of a thread keep their costs in registers for the second pass
-  constexpr int CACHED = 4;
-  uint64_t cc[CACHED];
   uint64_t c_min = ~uint64_t(0);
-#pragma unroll
-  for (int q = 0; q < CACHED; ++q) {
-    const int i = t + nt * q;
-    cc[q] = i < total ? plan_cost(p, n_mt, glo + i / nv, vlo + i % nv) : ~uint64_t(0);
-    c_min = cc[q] < c_min ? cc[q] : c_min;
-  }
-  for (int i = t + nt * CACHED; i < total; i += nt) {
+#pragma unroll 1
+  for (int i = t; i < total; i += nt) {
     const uint64_t c = plan_cost(p, n_mt, glo + i / nv, vlo + i % nv);
+    if (i < PlanScratch::KEPT) sh->cost[i] = c < 0xffffffffu ? static_cast<uint32_t>(c) : 0xffffffffu;
     c_min = c < c_min ? c : c_min;
   }
   c_min = cta_min(c_min, sh);
   const uint64_t c_max = c_min + c_min / MAKESPAN_SLACK_DIV;
   uint64_t best = ~uint64_t(0);
-#pragma unroll
-  for (int q = 0; q < CACHED; ++q) {
-    const int i = t + nt * q;
-    if (i < total && cc[q] <= c_max) {
-      const uint64_t k = plan_key(p, n_mt, glo + i / nv, vlo + i % nv, cc[q]);
-      best = k < best ? k : best;
-    }
-  }
-  for (int i = t + nt * CACHED; i < total; i += nt) {
-    const uint64_t c = plan_cost(p, n_mt, glo + i / nv, vlo + i % nv);
+#pragma unroll 1
+  for (int i = t; i < total; i += nt) {
+    uint64_t c = i < PlanScratch::KEPT ? sh->cost[i] : 0xffffffffu;  // this thread's own
+    if (c == 0xffffffffu) c = plan_cost(p, n_mt, glo + i / nv, vlo + i % nv);
     if (c > c_max) continue;
     const uint64_t k = plan_key(p, n_mt, glo + i / nv, vlo + i % nv, c);
     best = k < best ? k : best;

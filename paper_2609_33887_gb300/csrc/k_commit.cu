@@ -1,9 +1,10 @@
 // Merge of the per-part softmax partials and the threshold commit with the
 // per-block top-1 fallback, for every tau of the grid in one pass.
 //
-// One CTA (8 warps) per block of the window. Threads split the partial slots
-// of each masked position, warp 0 finishes the merge and then applies, for
-// every tau_k, the rule
+// One CTA of 32 warps per block of the window. A thread takes one position and
+// every 32nd (blocks longer than 32: every 16th) partial slot, its loads issued
+// together; a warp then merges a position's (or two positions') threads by
+// shuffles, and warp 0 applies, for every tau_k, the rule
 //   commit(p, k) = masked(p) && active(block) && conf(p) >= tau_k           (Sec. 3.1, App. B.1)
 //                  || the block is fallback-eligible, holds a masked position,
 //                     no position cleared tau_k, and p is the masked position of
@@ -21,32 +22,39 @@
 namespace bd {
 
 namespace {
-constexpr int THREADS = 256;
+constexpr int THREADS = 1024;
 constexpr int MAX_L = 64;
-constexpr int MAX_GROUPS = THREADS / 32;
+// Partial slots a thread loads at once. The kernel's bound is its chain of
+// latencies (header, row, partials, combines): it ends 3.8 us after the LM head
+// on the 8 x 2 x 32 window, 5.5 us with 256 threads that took nine slots each
+// and warp 0 merging eight groups per position.
+constexpr int BATCH = 4;
 }  // namespace
 
-template <int MODE>
+// LP: positions a CTA handles side by side, 32 or 64 (>= the block length)
+template <int MODE, int LP>
 __global__ void __launch_bounds__(THREADS) merge_commit_kernel(CommitArgs a) {
-  __shared__ float sm_m[MAX_GROUPS][MAX_L], sm_s[MAX_GROUPS][MAX_L];
-  __shared__ int sm_a[MAX_GROUPS][MAX_L];
-  __shared__ bool sm_live[MAX_L];  // the position has a compacted row (read once, in the merge stage)
+  constexpr int GROUPS = THREADS / LP;  // threads per position
+  // thread (group g, position j): [j][g], padded so that both directions hit different banks
+  __shared__ float sm_m[LP][GROUPS + 1], sm_s[LP][GROUPS + 1];
+  __shared__ int sm_a[LP][GROUPS + 1];
+  // the merged state of each position, and whether it has a compacted row
+  __shared__ float mg_m[LP], mg_s[LP];
+  __shared__ int mg_a[LP];
+  __shared__ bool sm_live[LP];
   const int blk = blockIdx.x;
   const int L = a.block_len;
   const int64_t base = static_cast<int64_t>(blk) * L;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  griddep_wait();  // the partials come from the LM-head kernel
+  griddep_launch_dependents();  // a kernel behind this one waits for it before touching memory
+  griddep_wait();               // the partials come from the LM-head kernel
   // partial slots per row over the plan's launches (header word)
   const int slots = MODE == MERGE_GATHERED ? a.n_parts : a.n_rows[HDR_SLOTS];
 
-  // ---- a3: merge of the partial slots. Thread t takes position t % Lp of the
-  // block and every groups-th slot starting at t / Lp; loads are issued four
-  // slots at a time so their latencies overlap.
-  const int Lp = L <= 32 ? 32 : 64;
-  const int groups = THREADS / Lp;
+  // ---- a3: merge of the partial slots
   {
-    const int jj = threadIdx.x % Lp;
-    const int g = threadIdx.x / Lp;
+    const int jj = threadIdx.x % LP;
+    const int g = threadIdx.x / LP;
     float m = -INFINITY, s = 0.f;
     int arg = 0x7fffffff;
     // partial slots the workspace holds (index checks of the bounds-checked build)
@@ -60,33 +68,45 @@ __global__ void __launch_bounds__(THREADS) merge_commit_kernel(CommitArgs a) {
       else
         r = a.rowpos[base + jj];
     }
+    if (g == 0) sm_live[jj] = r >= 0;
     if (r >= 0 && index_ok(r, a.P, a.status)) {
-      const int ns = slots;
-      int slot = g;
-      for (; slot + 3 * groups < ns; slot += 4 * groups) {
-        float pm[4], ps[4];
-        int pa[4];
+#pragma unroll 1
+      for (int slot = g; slot < slots; slot += BATCH * GROUPS) {
+        float pm[BATCH], ps[BATCH];
+        int pa[BATCH];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int64_t o = static_cast<int64_t>(slot + u * groups) * a.P + r;
-          const bool in = index_ok(o, part_n, a.status);
+        for (int u = 0; u < BATCH; ++u) {
+          const int64_t o = static_cast<int64_t>(slot + u * GROUPS) * a.P + r;
+          const bool in = slot + u * GROUPS < slots && index_ok(o, part_n, a.status);
           pm[u] = in ? a.part_m[o] : -INFINITY;
           ps[u] = in ? a.part_s[o] : 0.f;
           pa[u] = in ? a.part_a[o] : 0x7fffffff;
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) softmax_combine(m, s, arg, pm[u], ps[u], pa[u]);
-      }
-      for (; slot < ns; slot += groups) {
-        const int64_t o = static_cast<int64_t>(slot) * a.P + r;
-        if (index_ok(o, part_n, a.status)) softmax_combine(m, s, arg, a.part_m[o], a.part_s[o], a.part_a[o]);
+        for (int u = 0; u < BATCH; ++u) softmax_combine(m, s, arg, pm[u], ps[u], pa[u]);
       }
     }
-    if (jj < L) {
-      sm_m[g][jj] = m;
-      sm_s[g][jj] = s;
-      sm_a[g][jj] = arg;
-      if (g == 0) sm_live[jj] = r >= 0;
+    sm_m[jj][g] = m;
+    sm_s[jj][g] = s;
+    sm_a[jj][g] = arg;
+  }
+  __syncthreads();
+  {
+    // warp w: position w (LP = 32), or positions 2 w and 2 w + 1 in its half-warps (LP = 64)
+    const int jj = (threadIdx.x / GROUPS), g = threadIdx.x % GROUPS;
+    float m = sm_m[jj][g], s = sm_s[jj][g];
+    int arg = sm_a[jj][g];
+#pragma unroll
+    for (int o = GROUPS / 2; o > 0; o >>= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, m, o);
+      const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
+      const int a2 = __shfl_xor_sync(0xffffffffu, arg, o);
+      softmax_combine(m, s, arg, m2, s2, a2);
+    }
+    if (g == 0) {
+      mg_m[jj] = m;
+      mg_s[jj] = s;
+      mg_a[jj] = arg;
     }
   }
   __syncthreads();
@@ -95,17 +115,15 @@ __global__ void __launch_bounds__(THREADS) merge_commit_kernel(CommitArgs a) {
   if constexpr (MODE == MERGE_EMIT) {
     // one partial per window position, token ids of the whole vocabulary
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < LP / 32; ++h) {
       const int jj = lane + 32 * h;
       if (jj < L) {
         float m = -INFINITY, s = 0.f;
         int arg = -1;
         if (sm_live[jj]) {
-          m = sm_m[0][jj];
-          s = sm_s[0][jj];
-          arg = sm_a[0][jj];
-          for (int g = 1; g < groups; ++g) softmax_combine(m, s, arg, sm_m[g][jj], sm_s[g][jj], sm_a[g][jj]);
-          arg = m == -INFINITY ? -1 : arg + a.vocab_offset;  // a shard holding only the mask token: nothing
+          m = mg_m[jj];
+          s = mg_s[jj];
+          arg = m == -INFINITY ? -1 : mg_a[jj] + a.vocab_offset;  // a shard holding only the mask token: nothing
         }
         a.emit_m[base + jj] = m;
         a.emit_s[base + jj] = s;
@@ -117,21 +135,16 @@ __global__ void __launch_bounds__(THREADS) merge_commit_kernel(CommitArgs a) {
 
   const uint32_t flags = a.block_flags[blk];
   const bool eligible = (flags & 2u) != 0;
-  bool live[2];
-  float conf[2];
-  int tok[2];
+  bool live[2] = {false, false};
+  float conf[2] = {0.f, 0.f};
+  int tok[2] = {-1, -1};
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < LP / 32; ++h) {
     const int jj = lane + 32 * h;
     live[h] = jj < L && sm_live[jj];
-    conf[h] = 0.f;
-    tok[h] = -1;
     if (live[h]) {
-      float m = sm_m[0][jj], s = sm_s[0][jj];
-      int arg = sm_a[0][jj];
-      for (int g = 1; g < groups; ++g) softmax_combine(m, s, arg, sm_m[g][jj], sm_s[g][jj], sm_a[g][jj]);
-      conf[h] = 1.f / s;  // s >= 1: the maximum contributes exp(0)
-      tok[h] = arg;
+      conf[h] = 1.f / mg_s[jj];  // the sum is >= 1: the maximum contributes exp(0)
+      tok[h] = mg_a[jj];
     }
   }
 
@@ -204,13 +217,15 @@ cudaError_t launch_merge_commit(const CommitArgs& a, cudaStream_t st, int mode) 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  const bool wide = a.block_len > 32;
   switch (mode) {
     case MERGE_EMIT:
-      return cudaLaunchKernelEx(&cfg, merge_commit_kernel<MERGE_EMIT>, a);
+      return cudaLaunchKernelEx(&cfg, wide ? merge_commit_kernel<MERGE_EMIT, 64> : merge_commit_kernel<MERGE_EMIT, 32>, a);
     case MERGE_GATHERED:
-      return cudaLaunchKernelEx(&cfg, merge_commit_kernel<MERGE_GATHERED>, a);
+      return cudaLaunchKernelEx(
+          &cfg, wide ? merge_commit_kernel<MERGE_GATHERED, 64> : merge_commit_kernel<MERGE_GATHERED, 32>, a);
     default:
-      return cudaLaunchKernelEx(&cfg, merge_commit_kernel<MERGE_ROWS>, a);
+      return cudaLaunchKernelEx(&cfg, wide ? merge_commit_kernel<MERGE_ROWS, 64> : merge_commit_kernel<MERGE_ROWS, 32>, a);
   }
 }
 

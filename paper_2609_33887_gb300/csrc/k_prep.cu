@@ -20,7 +20,9 @@ namespace bd {
 // hidden rows of its live positions into hc (tensor-core paths), one warp per
 // row with the whole row's loads in flight.
 //
-// Bound: latency on small windows, where the LM head waits for this kernel.
+// Bound: latency on small windows, where the LM head waits for this kernel (an
+// 8 x 2 x 32 bf16 window: the header 2.8 us and the rows 3.5 us after its
+// start); HBM on large ones.
 // Chunks are therefore as small as eight positions (a row per warp) until the
 // grid has four CTAs per SM.
 // ---------------------------------------------------------------------------
@@ -200,7 +202,7 @@ __device__ __forceinline__ int64_t packed_row_bytes(int64_t ldc) {
 // One warp packs the d elements of the bf16 row src into dst (16-byte aligned
 // rows of row_bytes; ROWS_E4M3X2: the lo terms lo_offset bytes after the hi
 // terms) and returns the row's token scale.
-template <int FMT>
+template <int FMT, int RC>
 __device__ __forceinline__ float pack_row(const __nv_bfloat16* __restrict__ src, int d, uint8_t* __restrict__ dst,
                                           int64_t lo_offset) {
   const int lane = threadIdx.x & 31, nvec = d / 8;
@@ -212,8 +214,7 @@ __device__ __forceinline__ float pack_row(const __nv_bfloat16* __restrict__ src,
     for (int e = nvec * 8 + lane; e < d; e += 32) reinterpret_cast<__nv_bfloat16*>(dst)[e] = src[e];
     return 1.f;
   } else {
-    // rows of up to 32 * RC vectors (5120 bf16) are read once, into registers
-    constexpr int RC = 20;
+    // rows of up to 32 * RC vectors are read once, into registers
     const bool cached = nvec <= 32 * RC;
     uint4 qc[RC];
     float amax = 0.f;
@@ -252,7 +253,12 @@ __device__ __forceinline__ float pack_row(const __nv_bfloat16* __restrict__ src,
   }
 }
 
-template <int FMT>  // the packed row format (ROWS_*); one instantiation per format
+// FMT: the packed row format (ROWS_*). RC: vectors of a row a lane keeps in
+// registers: 8 for rows of up to 2048 elements, else 20 (5120). The straight
+// code for 20 costs a short row its instruction fetches: an 8 x 2 x 32 window's
+// E4M3X2 rows (d = 2048) were packed 7.5 us after the kernel's start with it,
+// 4.9 us without.
+template <int FMT, int RC>
 __global__ void __launch_bounds__(PREP_THREADS, 2) prep_rows_kernel(PrepArgs a) {
   __shared__ int red[2][PREP_WARPS];
   __shared__ int rows_s[PREP_MAX_CHUNK];
@@ -314,8 +320,8 @@ __global__ void __launch_bounds__(PREP_THREADS, 2) prep_rows_kernel(PrepArgs a) 
   for (int i = warp; i < local_total; i += PREP_WARPS) {
     const int r = prefix + i;
     if (!index_ok(r, a.P, a.status)) continue;
-    const float scale = pack_row<FMT>(a.hidden + static_cast<int64_t>(rows_s[i]) * a.ld, a.d,
-                                      static_cast<uint8_t*>(a.hc) + r * row_bytes, a.P * row_bytes);
+    const float scale = pack_row<FMT, RC>(a.hidden + static_cast<int64_t>(rows_s[i]) * a.ld, a.d,
+                                          static_cast<uint8_t*>(a.hc) + r * row_bytes, a.P * row_bytes);
     if (FMT != ROWS_BF16 && lane == 0) a.tok_scale[r] = scale;
   }
 }
@@ -352,10 +358,11 @@ cudaError_t launch_prep_rows(const PrepArgs& args, int row_format, int sm_count,
   PrepArgs a = args;
   a.chunk = prep_chunk(a.P, sm_count);
   const int grid = 1 + (a.P + a.chunk - 1) / a.chunk;
-  auto* kern = row_format == ROWS_F16_POW2 ? prep_rows_kernel<ROWS_F16_POW2>
-               : row_format == ROWS_E4M3  ? prep_rows_kernel<ROWS_E4M3>
-               : row_format == ROWS_E4M3X2 ? prep_rows_kernel<ROWS_E4M3X2>
-                                           : prep_rows_kernel<ROWS_BF16>;
+  const bool small = a.d <= 2048;
+  auto* kern = row_format == ROWS_F16_POW2 ? (small ? prep_rows_kernel<ROWS_F16_POW2, 8> : prep_rows_kernel<ROWS_F16_POW2, 20>)
+               : row_format == ROWS_E4M3   ? (small ? prep_rows_kernel<ROWS_E4M3, 8> : prep_rows_kernel<ROWS_E4M3, 20>)
+               : row_format == ROWS_E4M3X2 ? (small ? prep_rows_kernel<ROWS_E4M3X2, 8> : prep_rows_kernel<ROWS_E4M3X2, 20>)
+                                           : prep_rows_kernel<ROWS_BF16, 1>;
   return launch_behind(kern, grid, st, a);
 }
 
@@ -366,7 +373,7 @@ cudaError_t launch_prep_rows(const PrepArgs& args, int row_format, int sm_count,
 // caller's rows in place (ROWS_BF16 here: nothing to pack); an E4M3 head on
 // the 8-bit path reads them as two E4M3 terms, packed by one warp per row.
 // ---------------------------------------------------------------------------
-template <int FMT>
+template <int FMT, int RC>
 __global__ void __launch_bounds__(PREP_THREADS, 2) prep_verify_kernel(PrepVerifyArgs a) {
   __shared__ PlanScratch plan_s;
   griddep_launch_dependents();
@@ -385,8 +392,8 @@ __global__ void __launch_bounds__(PREP_THREADS, 2) prep_verify_kernel(PrepVerify
   if constexpr (FMT != ROWS_BF16) {
     const int64_t row_bytes = packed_row_bytes<FMT>(a.ldc);
     for (int r = cta * PREP_WARPS + static_cast<int>(threadIdx.x >> 5); r < R; r += ctas * PREP_WARPS) {
-      const float scale = pack_row<FMT>(a.hidden + static_cast<int64_t>(r) * a.ld, a.d,
-                                        static_cast<uint8_t*>(a.hc) + r * row_bytes, R * row_bytes);
+      const float scale = pack_row<FMT, RC>(a.hidden + static_cast<int64_t>(r) * a.ld, a.d,
+                                            static_cast<uint8_t*>(a.hc) + r * row_bytes, R * row_bytes);
       if ((threadIdx.x & 31) == 0) a.tok_scale[r] = scale;
     }
   }
@@ -399,8 +406,10 @@ cudaError_t launch_prep_verify(const PrepVerifyArgs& a, int row_format, cudaStre
   int grid = (R + rows - 1) / rows;
   if (grid < 1) grid = 1;
   if (grid > 1024) grid = 1024;
-  return row_format == ROWS_BF16 ? launch_behind(prep_verify_kernel<ROWS_BF16>, 1 + grid, st, a)
-                                 : launch_behind(prep_verify_kernel<ROWS_E4M3X2>, 1 + grid, st, a);
+  auto* kern = row_format == ROWS_BF16 ? prep_verify_kernel<ROWS_BF16, 1>
+               : a.d <= 2048           ? prep_verify_kernel<ROWS_E4M3X2, 8>
+                                       : prep_verify_kernel<ROWS_E4M3X2, 20>;
+  return launch_behind(kern, 1 + grid, st, a);
 }
 
 // ---------------------------------------------------------------------------

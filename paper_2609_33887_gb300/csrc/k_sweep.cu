@@ -43,7 +43,8 @@ __global__ void __launch_bounds__(SWEEP_THREADS) commit_sweep_kernel(SweepArgs a
 
   const int tid = threadIdx.x, B = a.n_slots, L = a.block_len, W = B * L;
   const int64_t base = static_cast<int64_t>(blockIdx.x) * W;
-  bd::griddep_wait();  // step_tokens / step_commit / the window come from the commit step
+  bd::griddep_launch_dependents();  // a kernel behind this one waits for it before touching memory
+  bd::griddep_wait();               // step_tokens / step_commit / the window come from the commit step
 
   if (tid < B) {
     n_masked[tid] = 0;
@@ -104,7 +105,6 @@ __global__ void __launch_bounds__(SWEEP_THREADS) commit_sweep_kernel(SweepArgs a
   }
   __syncthreads();
   if (tid < B) a.block_flags[static_cast<int64_t>(blockIdx.x) * B + tid] = new_flg[tid];
-  bd::griddep_launch_dependents();
 }
 
 // Compute capability check per device, cached (0 = unknown, 1 = sm_103, 2 = other).

@@ -24,7 +24,8 @@ __global__ void __launch_bounds__(THREADS) merge_verify_kernel(VerifyArgs a) {
   const int q = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int D = a.n_draft, Rq = D + 1;
-  griddep_wait();  // the partials come from the LM-head kernel
+  griddep_launch_dependents();  // a kernel behind this one waits for it before touching memory
+  griddep_wait();               // the partials come from the LM-head kernel
   // partial slots per row over the plan's launches (header word)
   const int ns = a.n_rows[HDR_SLOTS];
 
