@@ -52,8 +52,7 @@
 //
 // The verification instantiation (VERIFY = true, speculative decoding) also
 // carries, per token, the entropy accumulator sum exp(l - m) (l - m) log2(e)
-// and the logit of the token's draft entry (typical-acceptance appendix); its
-// larger combine buffers cost shared memory, so it may run one stage fewer.
+// and the logit of the token's draft entry (typical-acceptance appendix).
 //
 // W8A8 (HF = HF_W8A8): E4M3 head rows times E4M3 token rows (quantised per
 // row by the compaction kernel) with tcgen05.mma kind::f8f6f4, K = 32 per
@@ -195,36 +194,27 @@ struct PairCtl {
   int abort_flag;
 };
 
-// One buffer per epilogue warp: the 32 x 33 transpose during the tiles of a
-// unit; after the warp's last tile, the same warp's running states (max, sum,
-// argmax for up to 256 tokens; with VERIFY also the entropy accumulator and
-// the draft logit) for the cross-warp combine. A warp only ever writes its own
+// One buffer per epilogue warp, below the control block at the end of shared
+// memory: the 32 x 33 transpose during the tiles of a unit; after the warp's
+// last tile, the same warp's running states (max, sum, argmax of its group's
+// tokens; with VERIFY also the entropy accumulator and the draft logit) for the
+// cross-warp combine, a row of NT words each. A warp only ever writes its own
 // buffer before the rendezvous, so no warp can overwrite a buffer another warp
-// is still transposing in.
+// is still transposing in. Sized by NT, the verification path keeps the fourth
+// stage of a 160-row group: 64 x 5 rows, d = 4096, V = 128256 take 207 us, with
+// buffers for 256 tokens and three stages 241 us.
+enum : int { ST_M = 0, ST_S = 1, ST_A = 2, ST_T = 3, ST_X = 4 };
 template <bool VERIFY>
-struct PairWarpBuf {
-  union {
-    float tr[32 * TR];
-    struct {
-      float m[256];
-      float s[256];
-      int a[256];
-      float t[VERIFY ? 256 : 1];
-      float x[VERIFY ? 256 : 1];
-    } st;
-  };
-};
-
-template <bool VERIFY, int EW>
-struct PairTail {
-  PairWarpBuf<VERIFY> w[EW];
-  PairCtl ctl;
-};
+__host__ __device__ constexpr int buf_words(int nt) {
+  return (VERIFY ? 5 : 3) * nt > 32 * TR ? (VERIFY ? 5 : 3) * nt : 32 * TR;
+}
 
 constexpr size_t SMEM_BYTES = 232448;  // the whole opt-in shared memory of an SM
+constexpr size_t CTL_OFFSET = SMEM_BYTES - 1024 - sizeof(PairCtl);
+static_assert(CTL_OFFSET % 8 == 0, "barriers and transpose rows on 8-byte boundaries");
 template <int HF, bool VERIFY>
-__host__ __device__ constexpr size_t stage_area() {
-  return SMEM_BYTES - 1024 - sizeof(PairTail<VERIFY, epi_warps<HF>()>);
+__host__ __device__ constexpr size_t stage_area(int nt) {
+  return CTL_OFFSET - 4 * static_cast<size_t>(epi_warps<HF>() * buf_words<VERIFY>(nt));
 }
 
 // Stage layout for a token group of NT rows (NT/2 in each CTA), one block per
@@ -241,7 +231,7 @@ __host__ __device__ constexpr uint32_t stage_bytes(int nt) {
 // no more than the A stages in tensor memory, and at most QUANT_STAGES.
 template <int HF, bool VERIFY>
 __host__ __device__ constexpr int stage_count(int nt) {
-  int n = static_cast<int>((stage_area<HF, VERIFY>() - (is_quant<HF>() ? MIN_RAW * raw_bytes<HF>() : 0)) /
+  int n = static_cast<int>((stage_area<HF, VERIFY>(nt) - (is_quant<HF>() ? MIN_RAW * raw_bytes<HF>() : 0)) /
                            stage_bytes<HF>(nt));
   if (n > MAX_STAGES) n = MAX_STAGES;
   if (is_quant<HF>() && n > a_stages(nt)) n = a_stages(nt);
@@ -251,14 +241,14 @@ __host__ __device__ constexpr int stage_count(int nt) {
 template <int HF, bool VERIFY>
 __host__ __device__ constexpr int raw_count(int nt) {
   return !is_quant<HF>() ? 0
-         : static_cast<int>((stage_area<HF, VERIFY>() - stage_count<HF, VERIFY>(nt) * stage_bytes<HF>(nt)) /
+         : static_cast<int>((stage_area<HF, VERIFY>(nt) - stage_count<HF, VERIFY>(nt) * stage_bytes<HF>(nt)) /
                             raw_bytes<HF>()) < MAX_RAW
-             ? static_cast<int>((stage_area<HF, VERIFY>() - stage_count<HF, VERIFY>(nt) * stage_bytes<HF>(nt)) /
+             ? static_cast<int>((stage_area<HF, VERIFY>(nt) - stage_count<HF, VERIFY>(nt) * stage_bytes<HF>(nt)) /
                                 raw_bytes<HF>())
              : MAX_RAW;
 }
 static_assert(stage_count<HF_BF16, false>(256) >= 3 && stage_count<HF_BF16, true>(256) >= 3, "three stages at NT = 256");
-static_assert(stage_count<HF_BF16, false>(160) == 4, "four stages at NT = 160 on the commit path");
+static_assert(stage_count<HF_BF16, false>(160) == 4 && stage_count<HF_BF16, true>(160) == 4, "four stages at NT = 160");
 static_assert(stage_count<HF_W8A8, false>(160) == 7 && stage_count<HF_W8A8, false>(256) >= 5,
               "W8A8: seven 26 KB stages at NT = 160, five 32 KB stages at NT = 256");
 static_assert(stage_count<HF_E4M3X2, false>(160) == 5 && stage_count<HF_E4M3X2, false>(256) == 4,
@@ -347,8 +337,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   constexpr int EW = epi_warps<HF>();
-  PairTail<VERIFY, EW>* tail = reinterpret_cast<PairTail<VERIFY, EW>*>(smem + stage_area<HF, VERIFY>());
-  PairCtl* ctl = &tail->ctl;
+  PairCtl* ctl = reinterpret_cast<PairCtl*>(smem + CTL_OFFSET);
   const uint32_t smem_base = smem_u32(smem);
 
   // pairs per cluster: two sharing head tiles (mc = 2) or token rows (vc = 2)
@@ -711,7 +700,10 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     // with eight epilogue warps, warp ew takes the chunks c with c % 2 == ew / 4
     const int chunk_par = EW == 8 ? (ew >> 2) : -1;
     const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
-    float* tr = tail->w[ew].tr;
+    // warp w's buffer, and its row of running states `what`
+    auto buf = [&](int w) { return reinterpret_cast<float*>(smem + CTL_OFFSET) - (w + 1) * buf_words<VERIFY>(NT); };
+    auto st = [&](int w, int what) { return buf(w) + what * NT; };
+    float* tr = buf(ew);
     const uint32_t tempty_local0 = smem_u32(&ctl->tempty[0]);
     const uint32_t tempty_leader0 = mapa_shared(tempty_local0, lead);
     const uint32_t epi_sync = smem_u32(&ctl->epi_sync);
@@ -869,12 +861,12 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
 #pragma unroll
       for (int c = 0; c < MAX_CHUNKS; ++c) {
         if (c < nch && (chunk_par < 0 || (c & 1) == chunk_par)) {
-          tail->w[ew].st.m[c * 32 + lane] = TOKS ? m[c] * ts[c] : m[c];
-          tail->w[ew].st.s[c * 32 + lane] = s[c];
-          tail->w[ew].st.a[c * 32 + lane] = arg[c];
+          st(ew, ST_M)[c * 32 + lane] = TOKS ? m[c] * ts[c] : m[c];
+          st(ew, ST_S)[c * 32 + lane] = s[c];
+          st(ew, ST_A)[c * 32 + lane] = __int_as_float(arg[c]);
           if constexpr (VERIFY) {
-            tail->w[ew].st.t[c * 32 + lane] = t[c];
-            tail->w[ew].st.x[c * 32 + lane] = TOKS ? lx[c] * ts[c] : lx[c];
+            st(ew, ST_T)[c * 32 + lane] = t[c];
+            st(ew, ST_X)[c * 32 + lane] = TOKS ? lx[c] * ts[c] : lx[c];
           }
         }
       }
@@ -884,22 +876,22 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
       for (int j = ew * 32 + lane; j < NT; j += EW * 32) {
         // the four warps (one per lane quarter) that hold token j's states
         const int w0 = EW == 8 ? 4 * ((j >> 5) & 1) : 0;
-        float M = tail->w[w0].st.m[j], S = tail->w[w0].st.s[j];
-        int A = tail->w[w0].st.a[j];
+        float M = st(w0, ST_M)[j], S = st(w0, ST_S)[j];
+        int A = __float_as_int(st(w0, ST_A)[j]);
         float T = 0.f, LX = -INFINITY;
         if constexpr (VERIFY) {
-          T = tail->w[w0].st.t[j];
-          LX = tail->w[w0].st.x[j];
+          T = st(w0, ST_T)[j];
+          LX = st(w0, ST_X)[j];
         }
 #pragma unroll
         for (int q = 1; q < 4; ++q) {
           const int w = w0 + q;
           if constexpr (VERIFY) {
-            softmax_combine_t(M, S, A, T, tail->w[w].st.m[j], tail->w[w].st.s[j], tail->w[w].st.a[j],
-                              tail->w[w].st.t[j]);
-            LX = fmaxf(LX, tail->w[w].st.x[j]);
+            softmax_combine_t(M, S, A, T, st(w, ST_M)[j], st(w, ST_S)[j], __float_as_int(st(w, ST_A)[j]),
+                              st(w, ST_T)[j]);
+            LX = fmaxf(LX, st(w, ST_X)[j]);
           } else {
-            softmax_combine(M, S, A, tail->w[w].st.m[j], tail->w[w].st.s[j], tail->w[w].st.a[j]);
+            softmax_combine(M, S, A, st(w, ST_M)[j], st(w, ST_S)[j], __float_as_int(st(w, ST_A)[j]));
           }
         }
         const int row = (it.m_tile + pp_mt) * NT + j;
