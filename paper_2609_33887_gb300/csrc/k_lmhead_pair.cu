@@ -781,9 +781,10 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
             }
             __syncwarp();
             // this thread: token column c*32 + lane, vocabulary rows vrow0 + r
-            float cm = x[0];
+            float cm = max3(x[0], x[1], x[31]);
 #pragma unroll
-            for (int r = 1; r < 32; ++r) cm = fmaxf(cm, x[r]);
+            for (int r = 2; r < 30; r += 2) cm = max3(cm, x[r], x[r + 1]);
+            cm = fmaxf(cm, x[30]);
             if (cm > m[c]) {
               int rr = 31;
 #pragma unroll
@@ -824,21 +825,22 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
                 s[c] += s0 + s1;
                 t[c] += t0 + t1;
               } else {
-                float s0 = 0.f, s1 = 0.f;
+                float2 sum = make_float2(0.f, 0.f);
                 if (!wide) {
+                  const float2 kk = make_float2(k2[c], k2[c]), nmc = make_float2(-mc, -mc);
 #pragma unroll
                   for (int r = 0; r < 32; r += 2) {
-                    s0 += ex2_approx(fmaf(x[r], k2[c], -mc));
-                    s1 += ex2_approx(fmaf(x[r + 1], k2[c], -mc));
+                    const float2 u = fma2(make_float2(x[r], x[r + 1]), kk, nmc);
+                    sum = add2(sum, make_float2(ex2_approx(u.x), ex2_approx(u.y)));
                   }
                 } else {
 #pragma unroll
                   for (int r = 0; r < 32; r += 2) {
-                    s0 += ex2_approx((x[r] - m[c]) * k2[c]);
-                    s1 += ex2_approx((x[r + 1] - m[c]) * k2[c]);
+                    sum.x += ex2_approx((x[r] - m[c]) * k2[c]);
+                    sum.y += ex2_approx((x[r + 1] - m[c]) * k2[c]);
                   }
                 }
-                s[c] += s0 + s1;
+                s[c] += sum.x + sum.y;
               }
             }
           }
