@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     if (threadIdx.x == 0) atomicOr(a.status, DEV_BAD_LAUNCH);
     return;
   }
-  const int warp = threadIdx.x >> 5;
+  const int warp = static_cast<int>(warp_uniform(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   const uint32_t crank = cluster_ctarank();
   const uint32_t rank = crank & 1u;  // 0: the CTA that issues the pair's MMAs
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   tc_fence_before();
   cluster_sync_all();  // barriers initialised and TMEM allocated in both CTAs
   tc_fence_after();
-  const uint32_t tmem_base = ctl->tmem_base;
+  const uint32_t tmem_base = warp_uniform(ctl->tmem_base);
   volatile int* abort_flag = &ctl->abort_flag;
 
   // The packed rows and the header (N, the plan) come from the preceding
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   const bool spill = a.plan.role == 1;
   if (!spill) griddep_wait();
   if (!spill && a.plan.G2 > 0) griddep_launch_dependents();
-  const int n_rows = hdr_word(a.n_rows, HDR_N);
+  const int n_rows = static_cast<int>(warp_uniform(static_cast<uint32_t>(hdr_word(a.n_rows, HDR_N))));
   const int VC = plan_vc(plan_resolve(a.plan, n_rows));
   const int pp_mt = VC == 1 ? pp : 0;  // this pair's token group within the runner's m-tiles
   constexpr int BK = STAGE_K;
