@@ -1201,6 +1201,8 @@ int bd_verify_step(const bd_hidden* hidden, const bd_weight* weight, const bd_dr
       if ((rc = check_verify(hidden, weight, draft, eps, variant, &vc, false)) != BD_OK) return rc;
       plan = make_plan(vc.c, ctx->sm_count, ctx->pairs, ctx->quads);
       lay = make_verify_layout(vc.c, plan);
+      if (exec->workspace_bytes < lay.total && shrink_plan(vc.c, ctx->sm_count, &plan))
+        lay = make_verify_layout(vc.c, plan);
     }
   }
   uint8_t* ws = nullptr;

@@ -146,3 +146,23 @@ def test_verify_with_the_workspace_of_rows_read_in_place(monkeypatch):
         got = bdc.verify_step(h, w, draft, n_req, D, [0.3], weight_scale=scale, workspace=ws)
         assert torch.equal(got["tokens"], want["tokens"]) and torch.equal(got["accepted"], want["accepted"])
         assert float((got["p_draft"] - want["p_draft"]).abs().max()) < 4e-4
+
+
+def test_verify_with_the_workspace_of_a_decoded_copy(monkeypatch):
+    # more rows than vocabulary entries: the packed rows need more room than
+    # the head's bf16 copy, beside which only the slots of shared head tiles fit
+    n_req, D, d, V = 60, 4, 336, 200
+    h, w, scale, logit = make("e4m3", n_req * (D + 1), V, d, 5)
+    draft = logit.argmax(1).view(n_req, D + 1)[:, :D].int().reshape(-1).contiguous()
+    want = bdc.verify_step(h, w, draft, n_req, D, [0.3], weight_scale=scale)
+    monkeypatch.setenv("BD_FUSED_DECODE", "0")
+    monkeypatch.setenv("BD_E4M3_SPLIT", "0")
+    monkeypatch.setenv("BD_PAIR_MC", "2")
+    least = bdc.bd_verify_workspace_size(h, w, scale, draft, n_req, D, [0.3])
+    monkeypatch.delenv("BD_E4M3_SPLIT")
+    monkeypatch.delenv("BD_PAIR_MC")
+    ws = torch.empty(least + 256, dtype=torch.uint8, device="cuda")
+    ws = ws[(-ws.data_ptr()) % 256:][:least]
+    got = bdc.verify_step(h, w, draft, n_req, D, [0.3], weight_scale=scale, workspace=ws)
+    assert torch.equal(got["tokens"], want["tokens"]) and torch.equal(got["accepted"], want["accepted"])
+    assert float((got["p_draft"] - want["p_draft"]).abs().max()) < 4e-4
