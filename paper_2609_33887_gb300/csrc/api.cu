@@ -240,6 +240,31 @@ int64_t head_operand_bytes(const Call& c) {
   return c.d * esize(c.wdt);
 }
 
+// Vocabulary entries per tile of the SIMT kernel (32, 64, 112 or 128). N is
+// only known on the device, so the narrow tiles are chosen for half the row
+// groups (of 96) the window may hold: 32 entries up to a tile per SM (per
+// runner for verification), 64 up to 1.5 per SM (not for verification, which
+// has two CTAs per SM). LM head, float32, 128 / 112 / 64 / 32 entries: 15 rows,
+// d = 256, V = 4096 19.5 / 19.5 / 19.5 / 16.4 us; d = 512, 75 rows, V = 5000
+// 47 / 45 / 39 / 53, V = 12000 60 / 54 / 47 / 76, V = 20000 70 / 68 / 93 / 131,
+// 250 rows, V = 12000 100 / 93 / 111 / 228. Verification, 15 rows, V = 5000
+// 29 / 28 / 28 / 24, 75 rows, V = 12000 53 / 55 / 66 / 72. Of the wide ones the
+// width whose tiles on the SM with most of them are fewer entries, summed over
+// the groups the window may come to: V = 50304, 75 rows 117 / 107, 500 rows
+// 611 / 625; V = 9000, 500 rows 144 / 148, 1000 rows 277 / 234.
+int simt_tile(const Call& c, int sm_count) {
+  const int64_t groups = std::min<int64_t>((c.P + 95) / 96, 8), half = ((c.P + 95) / 96 + 1) / 2;
+  const auto tiles = [&c](int64_t g, int bn) { return g * ((c.V + bn - 1) / bn); };
+  if (tiles(half, 32) <= (c.verify ? bd::SIMT_CTAS_VERIFY : 1) * sm_count) return 32;
+  if (!c.verify && 2 * tiles(half, 64) <= 3 * sm_count) return 64;
+  int64_t narrow = 0, wide = 0;
+  for (int64_t g = 1; g <= groups; ++g) {
+    narrow += (tiles(g, 112) + sm_count - 1) / sm_count * 112;
+    wide += (tiles(g, 128) + sm_count - 1) / sm_count * 128;
+  }
+  return narrow < wide ? 112 : 128;
+}
+
 BandPlan make_plan(const Call& c, int sm_count, int pairs, int quads) {
   BandPlan p{};
   p.mc = 1;
@@ -287,11 +312,9 @@ BandPlan make_plan(const Call& c, int sm_count, int pairs, int quads) {
     p.G = sm_count;
     p.cpu = 1;
   } else {
-    // tiles of 128 entries unless the window (in groups of 96 rows) then has
-    // fewer than two tiles per SM
     p.BM = bd::BM_SIMT;
-    p.BN = (c.P + 95) / 96 * ((c.V + bd::SIMT_BN - 1) / bd::SIMT_BN) < 2 * sm_count ? bd::SIMT_BN_SMALL : bd::SIMT_BN;
     p.G = (c.verify ? bd::SIMT_CTAS_VERIFY : bd::SIMT_CTAS) * sm_count;
+    p.BN = simt_tile(c, sm_count);
     p.cpu = 1;
   }
   // bands: GM derived on the device from the head and row bytes (0), or fixed

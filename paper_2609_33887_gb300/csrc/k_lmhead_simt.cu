@@ -13,14 +13,15 @@
 // at one column hit different banks), filled by 16-byte asynchronous copies
 // into a ring of stages that runs on across the tiles of a unit.
 //
-// C = 8 is bound by instruction issue on the SMs that hold most tiles (77
-// rows, d = 1024, V = 50304: 393 tiles on 152 SMs, 36 TFLOP/s; FMAs are 78% of
-// its instructions, shared memory a third busy): 18 reads of four columns of d
-// feed 320 products of a thread. With one column of eight rows per thread the
-// same LM head took 520 us instead of 223 us, bound by nine reads per eight
-// products. C = 2 serves vocabularies that would leave most SMs without a tile
-// of 128 entries, with more, smaller stages in flight (32 rows, d = 256,
-// V = 4096: 19 us, latency).
+// C = 8 and 7 are bound by instruction issue on the SMs that hold most tiles
+// (FMAs are 78% of the instructions, shared memory a third busy): 18 reads of
+// four columns of d feed 320 products of a thread. 77 rows, d = 1024, V =
+// 50304: 201 us with C = 7 (450 tiles on 152 SMs), 223 us with C = 8 (393 tiles,
+// so the SMs with three of them set the time of all). With one column of eight
+// rows per thread the same LM head took 520 us, bound by nine reads per eight
+// products. C = 2 and 4 serve vocabularies that would leave most SMs without a
+// wider tile, with more, smaller stages in flight (32 rows, d = 256, V = 4096:
+// 17 us, latency). The host chooses C (simt_tile).
 #include <atomic>
 #include <cuda_fp16.h>
 
@@ -39,7 +40,7 @@ constexpr int MAX_R = 12;
 template <int C>
 __host__ __device__ constexpr int bn_of() { return 16 * C; }  // entries per tile
 template <int C>
-__host__ __device__ constexpr int stages_of() { return C == 8 ? 3 : 6; }
+__host__ __device__ constexpr int stages_of() { return C > 4 ? 3 : C == 4 ? 4 : 6; }
 template <bool VERIFY>
 __host__ __device__ constexpr int ctas_of() { return VERIFY ? SIMT_CTAS_VERIFY : SIMT_CTAS; }
 
@@ -363,9 +364,13 @@ static cudaError_t launch_simt(const SimtArgs& a, cudaStream_t st) {
 
 cudaError_t launch_lmhead_simt(const SimtArgs& a, cudaStream_t st) {
   const bool verify = a.part_t != nullptr;
-  if (a.plan.BN == bn_of<2>()) return verify ? launch_simt<2, true>(a, st) : launch_simt<2, false>(a, st);
-  if (a.plan.BN != bn_of<8>()) return cudaErrorInvalidValue;
-  return verify ? launch_simt<8, true>(a, st) : launch_simt<8, false>(a, st);
+  switch (a.plan.BN) {
+    case bn_of<2>(): return verify ? launch_simt<2, true>(a, st) : launch_simt<2, false>(a, st);
+    case bn_of<4>(): return verify ? cudaErrorInvalidValue : launch_simt<4, false>(a, st);
+    case bn_of<7>(): return verify ? launch_simt<7, true>(a, st) : launch_simt<7, false>(a, st);
+    case bn_of<8>(): return verify ? launch_simt<8, true>(a, st) : launch_simt<8, false>(a, st);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace bd

@@ -145,9 +145,8 @@ struct SimtArgs {
   float* part_t = nullptr;
   float* part_x = nullptr;
 };
-constexpr int SIMT_BN = 128;       // vocabulary entries per tile
-constexpr int SIMT_BN_SMALL = 32;  // ... where those would leave most SMs without one
-// CTAs per SM (plan.G = this times the SMs; plan.BM = BM_SIMT)
+// CTAs per SM (plan.G = this times the SMs; plan.BM = BM_SIMT; plan.BN = the
+// vocabulary entries per tile: 32, 112 or 128, or 64 outside verification)
 constexpr int SIMT_CTAS = 3, SIMT_CTAS_VERIFY = 2;
 cudaError_t launch_lmhead_simt(const SimtArgs& a, cudaStream_t st);
 

@@ -1,5 +1,5 @@
 """The float32 LM head at the edges of its tiles: row counts around its groups of 8 R rows, vocabularies around its
-tiles of 32 and 128 entries, widths around its 16-column stages, row strides and base addresses with no more than the
+tiles of 32, 64, 112 and 128 entries, widths around its 16-column stages, row strides and base addresses with no more than the
 4-byte alignment the entry points ask for, and a workspace without room for every runner's partials. Compared with a
 float64 evaluation of every position.
 """
@@ -45,7 +45,8 @@ TOL = 2e-4
 
 @pytest.mark.parametrize("N", [1, 7, 8, 9, 33, 40, 63, 64, 65, 77, 129, 200])
 @pytest.mark.parametrize("V,d,pad", [(5, 1, 0), (31, 15, 2), (33, 16, 0), (257, 17, 3), (4096, 100, 1),
-                                     (39000, 20, 0), (40001, 33, 5)])
+                                     (39000, 20, 0), (40001, 33, 5), (9001, 100, 1), (9024, 20, 0),
+                                     (17024, 16, 0), (17026, 33, 3), (19001, 15, 0), (19456, 20, 0)])
 def test_commit_step(N, V, d, pad):
     g = torch.Generator(device="cuda").manual_seed(N * V + d)
     h, w = strided(N, d, pad, g), strided(V, d, pad, g) / max(1, d) ** 0.5 * 2
@@ -59,7 +60,7 @@ def test_commit_step(N, V, d, pad):
 
 
 @pytest.mark.parametrize("n_req", [1, 9, 13, 40])  # 5, 45, 65 and 200 rows
-@pytest.mark.parametrize("V,d", [(33, 16), (4096, 100), (39000, 20)])
+@pytest.mark.parametrize("V,d", [(33, 16), (4096, 100), (39000, 20), (19001, 33), (17024, 20)])
 def test_verify_step(n_req, V, d):
     D, g = 4, torch.Generator(device="cuda").manual_seed(n_req + V)
     h, w = strided(n_req * (D + 1), d, 1, g), strided(V, d, 0, g) / d ** 0.5 * 2
