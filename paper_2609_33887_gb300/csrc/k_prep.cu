@@ -25,27 +25,32 @@ namespace bd {
 // start); HBM on large ones.
 // Chunks are therefore as small as eight positions (a row per warp) until the
 // grid has four CTAs per SM.
+//
+// The grid may be resident while the kernel before it still runs, and that
+// kernel may write what this one reads (the sweep moves the window on in
+// place): mask, flags and rows are read with plain loads behind griddep_wait,
+// never through the read-only path (ld.global.nc holds only for memory that
+// nobody writes during the kernel), and no pointer to them is __restrict__.
 // ---------------------------------------------------------------------------
 constexpr int PREP_THREADS = 256;
 constexpr int PREP_WARPS = PREP_THREADS / 32;
 constexpr int PREP_MAX_CHUNK = 2048;
 
-__device__ __forceinline__ int live_at(const uint8_t* __restrict__ pos_masked, const uint8_t* __restrict__ block_flags,
-                                       int p, int block_len) {
+__device__ __forceinline__ int live_at(const uint8_t* pos_masked, const uint8_t* block_flags, int p, int block_len) {
   return (pos_masked[p] != 0 && (block_flags[p / block_len] & 1u)) ? 1 : 0;
 }
 
 // This thread's share of the live positions in [0, n): 16 mask bytes per load
 // where the array starts on a 16-byte boundary.
-__device__ __forceinline__ int count_live(const uint8_t* __restrict__ pos_masked,
-                                          const uint8_t* __restrict__ block_flags, int n, int block_len) {
+__device__ __forceinline__ int count_live(const uint8_t* pos_masked, const uint8_t* block_flags, int n,
+                                          int block_len) {
   int cnt = 0;
   int done = 0;
   if ((reinterpret_cast<uintptr_t>(pos_masked) & 15u) == 0) {
     const int nv = n / 16;
     const uint4* m4 = reinterpret_cast<const uint4*>(pos_masked);
     for (int v = threadIdx.x; v < nv; v += PREP_THREADS) {
-      const uint4 q = __ldg(m4 + v);
+      const uint4 q = m4[v];
       const uint32_t w[4] = {q.x, q.y, q.z, q.w};
       int b = 16 * v / block_len;
       int rem = 16 * v - b * block_len;  // position within block b
@@ -201,16 +206,24 @@ __device__ __forceinline__ int64_t packed_row_bytes(int64_t ldc) {
 
 // One warp packs the d elements of the bf16 row src into dst (16-byte aligned
 // rows of row_bytes; ROWS_E4M3X2: the lo terms lo_offset bytes after the hi
-// terms) and returns the row's token scale.
+// terms) and returns the row's token scale. Loads are issued ahead of the
+// stores batch by batch: src and dst might alias for all the compiler knows.
 template <int FMT, int RC>
-__device__ __forceinline__ float pack_row(const __nv_bfloat16* __restrict__ src, int d, uint8_t* __restrict__ dst,
-                                          int64_t lo_offset) {
+__device__ __forceinline__ float pack_row(const __nv_bfloat16* src, int d, uint8_t* dst, int64_t lo_offset) {
   const int lane = threadIdx.x & 31, nvec = d / 8;
   const uint4* s4 = reinterpret_cast<const uint4*>(src);
   if constexpr (FMT == ROWS_BF16) {
+    constexpr int BATCH = 8;
     uint4* d4 = reinterpret_cast<uint4*>(dst);
-#pragma unroll 8
-    for (int v = lane; v < nvec; v += 32) d4[v] = __ldg(s4 + v);
+    for (int v0 = lane; v0 < nvec; v0 += 32 * BATCH) {
+      uint4 q[BATCH];
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k)
+        if (v0 + 32 * k < nvec) q[k] = s4[v0 + 32 * k];
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k)
+        if (v0 + 32 * k < nvec) d4[v0 + 32 * k] = q[k];
+    }
     for (int e = nvec * 8 + lane; e < d; e += 32) reinterpret_cast<__nv_bfloat16*>(dst)[e] = src[e];
     return 1.f;
   } else {
@@ -222,13 +235,13 @@ __device__ __forceinline__ float pack_row(const __nv_bfloat16* __restrict__ src,
 #pragma unroll
       for (int k = 0; k < RC; ++k) {
         const int v = lane + 32 * k;
-        qc[k] = v < nvec ? __ldg(s4 + v) : make_uint4(0u, 0u, 0u, 0u);
+        qc[k] = v < nvec ? s4[v] : make_uint4(0u, 0u, 0u, 0u);
       }
 #pragma unroll
       for (int k = 0; k < RC; ++k) amax = fmaxf(amax, amax8(qc[k]));
     } else {
 #pragma unroll 4
-      for (int v = lane; v < nvec; v += 32) amax = fmaxf(amax, amax8(__ldg(s4 + v)));
+      for (int v = lane; v < nvec; v += 32) amax = fmaxf(amax, amax8(s4[v]));
     }
     for (int e = nvec * 8 + lane; e < d; e += 32) amax = fmaxf(amax, fabsf(__bfloat162float(src[e])));
 #pragma unroll
@@ -245,8 +258,16 @@ __device__ __forceinline__ float pack_row(const __nv_bfloat16* __restrict__ src,
         if (v < nvec) out.store8(qc[k], v);
       }
     } else {
-#pragma unroll 4
-      for (int v = lane; v < nvec; v += 32) out.store8(__ldg(s4 + v), v);
+      constexpr int BATCH = 4;
+      for (int v0 = lane; v0 < nvec; v0 += 32 * BATCH) {
+        uint4 q[BATCH];
+#pragma unroll
+        for (int k = 0; k < BATCH; ++k)
+          if (v0 + 32 * k < nvec) q[k] = s4[v0 + 32 * k];
+#pragma unroll
+        for (int k = 0; k < BATCH; ++k)
+          if (v0 + 32 * k < nvec) out.store8(q[k], v0 + 32 * k);
+      }
     }
     for (int e = nvec * 8 + lane; e < d; e += 32) out.store1(__bfloat162float(src[e]), e);
     return scale;
