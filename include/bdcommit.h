@@ -166,11 +166,12 @@ typedef struct {
  *                     for timing it alone.
  *   variant         : 0 = automatic: the CTA-pair tensor-core kernel for BF16
  *                     heads at every window size and for E4M3 heads with
- *                     16-byte aligned rows (see below), and for NVFP4 heads whose
- *                     codes and block scales it can read as stored; quantised
- *                     heads it cannot read so on the CTA-pair kernel up to 8192
- *                     window positions and the one-CTA kernel above, on a decoded
- *                     bf16 copy; the fp32 SIMT kernel for F32 heads. 1 = force the fp32-FMA SIMT LM-head kernel; 2 =
+ *                     16-byte aligned rows (see below); NVFP4 heads whose codes and
+ *                     block scales it can read as stored on the CTA-pair kernel up
+ *                     to 16384 window positions (8192 verification rows) and the
+ *                     one-CTA kernel on a decoded bf16 copy above; quantised heads
+ *                     it cannot read so, decoded to a bf16 copy, with the line at
+ *                     8192; the fp32 SIMT kernel for F32 heads. 1 = force the fp32-FMA SIMT LM-head kernel; 2 =
  *                     force the one-CTA tensor-core kernel (tokens on the MMA M
  *                     side); 3 = force the CTA-pair tensor-core kernel
  *                     (vocabulary on the M side). 2 and 3 need BF16 hidden
@@ -269,8 +270,8 @@ int bd_plan_header(const bd_hidden* hidden, const bd_weight* weight, const bd_ma
  *   BD_FUSED_DECODE=0    quantised heads decoded to a bf16 copy, not in the kernel
  *   BD_PAIR_MAX_P=n      the automatic choice takes the CTA-pair kernel for
  *                        quantised heads off the 8-bit path up to n window
- *                        positions (default: always for heads decoded in the
- *                        kernel, 8192 on a decoded copy)
+ *                        positions (default: 16384 for commit steps whose
+ *                        head the kernel decodes itself, else 8192)
  *   BD_PAIR_MC=1|2       single CTA pairs, or clusters of two pairs sharing each
  *                        head tile by multicast (default: clusters for windows of
  *                        at most 512 positions or more than 256 MiB of packed rows)

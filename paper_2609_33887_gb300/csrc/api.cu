@@ -22,6 +22,11 @@ constexpr int MAX_DEVICES = 64;
 constexpr int64_t MAX_POSITIONS = int64_t(1) << 24;
 constexpr int64_t MAX_VOCAB = int64_t(1) << 30;
 constexpr int64_t MAX_DIM = int64_t(1) << 20;
+// Window positions up to which the automatic choice runs a quantised head off
+// the 8-bit path on the CTA-pair kernel (see check_head): a commit step whose
+// codes the kernel decodes itself, and the others.
+constexpr int PAIR_MAX_DECODED = 16384;
+constexpr int PAIR_MAX = 8192;
 
 struct DevCtx {
   bool ready = false;
@@ -85,6 +90,7 @@ struct Call {
   int64_t ldc;      // packed hidden rows (bf16), elements
   int64_t ldq;      // decoded e4m3 head (bf16), elements
   bool fused;       // pair kernel decodes an E4M3 / NVFP4 head itself (no bf16 copy)
+  bool either = false;   // a head both the pair kernel (fused) and the one-CTA kernel (a copy) may take
   bool fp8_act = false;  // W8A8: token rows quantised to E4M3, kind::f8f6f4 MMAs on the E4M3 head
   bool verify = false;   // verification rows (bd_verify_step)
   bool split = false;    // W8A16 on the 8-bit path: bf16 rows as two E4M3 terms times the E4M3 head
@@ -120,7 +126,7 @@ int env_int(const char* name, int dflt, int lo, int hi);
 // Checks shared by every entry point that runs the LM head: the head and the
 // `rows` hidden rows, their dtypes and alignment, and the kernel choice. Fills
 // the head fields of *c (d, V, dtypes, tc / pair, leading dimensions).
-int check_head(const bd_hidden* h, const bd_weight* w, int64_t rows, int variant, Call* c) {
+int check_head(const bd_hidden* h, const bd_weight* w, int64_t rows, int variant, Call* c, bool verify = false) {
   if (w->vocab < 1 || w->vocab > MAX_VOCAB) return BD_ERR_SHAPE;
   if (w->dim < 1 || w->dim > MAX_DIM || h->cols != w->dim) return BD_ERR_SHAPE;
   if (h->ld < h->cols || w->ld < (w->dtype == BD_NVFP4 ? (w->dim + 1) / 2 : w->dim)) return BD_ERR_SHAPE;
@@ -157,18 +163,23 @@ int check_head(const bd_hidden* h, const bd_weight* w, int64_t rows, int variant
                         (wdt != BD_NVFP4 || (aligned(w->block_scale, 16) && w->block_ld % 16 == 0));
   // automatic choice: the CTA-pair kernel (vocabulary on M, token dimension
   // padded only to a multiple of 32, 256 x 256 tiles per pair at large
-  // windows) for every head it reads as stored (NVFP4, d = 2048, V = 151936:
-  // 3.17 against 3.49 ms a step at 9000 positions and 5.72 against 5.92 ms at
-  // 16384 with the one-CTA kernel on a decoded bf16 copy, which costs 0.2 ms);
-  // on a decoded copy only while the window is small (at large windows the
-  // one-CTA kernel keeps the tensor pipe busier)
-  const int max_p = env_int("BD_PAIR_MAX_P", readable ? 1 << 30 : 8192, 0, 1 << 30);
+  // windows) for bf16 heads; for quantised ones while the window is small (at
+  // large windows the one-CTA kernel on a decoded bf16 copy, which costs 0.2
+  // ms, keeps the tensor pipe busier). Steps on the pair kernel decoding NVFP4
+  // codes itself against the one-CTA kernel, d = 2048 and V = 151936: 3.18 /
+  // 3.54 ms at 9000 positions, 5.73 / 5.99 at 16384, 12.05 / 11.79 at 32768,
+  // 24.5 / 23.7 at 65536; d = 4096 and V = 32000: 1.49 / 1.46, 2.73 / 2.67,
+  // 4.98 / 5.21 and 9.90 / 9.71 ms. Verification (bf16 operands, a longer
+  // epilogue), d = 4096 and V = 128256: 6.08 / 5.66 ms at 9000 rows, 11.6 /
+  // 10.3 at 16384; an E4M3 head 6.36 / 5.50 and 12.6 / 10.1 ms.
+  const int max_p = env_int("BD_PAIR_MAX_P", readable && !verify ? PAIR_MAX_DECODED : PAIR_MAX, 0, 1 << 30);
   c->pair = tc && (variant == 3 || (variant == 0 && (!quant_head || rows <= max_p)));
   c->ldh = h->ld;
   c->ldw = w->ld;
   c->ldc = round_up(c->d, 8);
   c->ldq = round_up(c->d, 8);
   c->fused = c->pair && readable;
+  c->either = tc && variant == 0 && readable && rows > PAIR_MAX;
   return BD_OK;
 }
 
@@ -367,10 +378,22 @@ bool shrink_plan(const Call& c, int sm_count, BandPlan* p) {
   return plan_max_slots(*p) < slots;
 }
 
-// The plan and layout for a workspace of `bytes`.
-Layout fit_layout(const Call& c, BandPlan* p, int sm_count, size_t bytes) {
-  Layout l = make_layout(c, *p);
-  if (l.total > bytes && shrink_plan(c, sm_count, p)) l = make_layout(c, *p);
+// The plan and layout of a call in a workspace of `bytes` (too large a layout
+// if it does not fit). Above PAIR_MAX positions a quantised head that does
+// not fit on its kernel goes to the other one if that does: the pair kernel
+// decoding it (two partials per vocabulary part and row) or the one-CTA kernel
+// (one, and the decoded copy).
+template <typename F>
+auto fit_call(Call* c, BandPlan* p, int sm_count, int pairs, int quads, size_t bytes, F layout)
+    -> decltype(layout(*c, *p)) {
+  *p = make_plan(*c, sm_count, pairs, quads);
+  auto l = layout(*c, *p);
+  if (l.total > bytes && shrink_plan(*c, sm_count, p)) l = layout(*c, *p);
+  if (l.total > bytes && c->either && !c->split && !c->fp8_act) {
+    c->pair = c->fused = !c->fused;
+    *p = make_plan(*c, sm_count, pairs, quads);
+    l = layout(*c, *p);
+  }
   return l;
 }
 
@@ -738,8 +761,9 @@ int bd_commit_step_ex(const bd_hidden* hidden, const bd_weight* weight, const bd
   DevCtx* ctx = nullptr;
   rc = device_ctx(&ctx);
   if (rc != BD_OK) return rc;
-  BandPlan plan = make_plan(c, ctx->sm_count, ctx->pairs, ctx->quads);
-  const Layout lay = fit_layout(c, &plan, ctx->sm_count, exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX);
+  BandPlan plan;
+  const Layout lay = fit_call(&c, &plan, ctx->sm_count, ctx->pairs, ctx->quads,
+                              exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX, make_layout);
 
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {
@@ -793,8 +817,9 @@ int bd_lmhead_partials(const bd_hidden* hidden, const bd_weight* shard, int64_t 
   DevCtx* ctx = nullptr;
   rc = device_ctx(&ctx);
   if (rc != BD_OK) return rc;
-  BandPlan plan = make_plan(c, ctx->sm_count, ctx->pairs, ctx->quads);
-  const Layout lay = fit_layout(c, &plan, ctx->sm_count, exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX);
+  BandPlan plan;
+  const Layout lay = fit_call(&c, &plan, ctx->sm_count, ctx->pairs, ctx->quads,
+                              exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX, make_layout);
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {
     if (exec->workspace_bytes < lay.total) return BD_ERR_WORKSPACE;
@@ -1005,8 +1030,9 @@ extern "C" int bd_commit_step_static(const bd_hidden* hidden, const bd_weight* w
   StaticCtx* sctx = nullptr;
   rc = static_ctx(&sctx);
   if (rc != BD_OK) return rc;
-  BandPlan plan = make_plan(c, sctx->sm_count, sctx->pairs, sctx->quads);
-  const Layout lay = fit_layout(c, &plan, sctx->sm_count, BD_STATIC_SCRATCH_BYTES);
+  BandPlan plan;
+  const Layout lay =
+      fit_call(&c, &plan, sctx->sm_count, sctx->pairs, sctx->quads, BD_STATIC_SCRATCH_BYTES, make_layout);
   if (lay.total > BD_STATIC_SCRATCH_BYTES) return BD_ERR_WORKSPACE;
 
   uint8_t* ws = sctx->scratch;
@@ -1071,7 +1097,7 @@ int check_verify(const bd_hidden* h, const bd_weight* w, const bd_draft* dr, con
   if (R > MAX_POSITIONS || h->rows != R) return BD_ERR_SHAPE;
   Call& c = vc->c;
   c = Call{};
-  if (const int rc = check_head(h, w, R, variant, &c)) return rc;
+  if (const int rc = check_head(h, w, R, variant, &c, true)) return rc;
   if (R > 0 && !dr->draft) return BD_ERR_NULL;
   if (R > 0 && !aligned(dr->draft, 4)) return BD_ERR_ALIGN;
   if (allow_split) choose_split(w, variant, &c);
@@ -1215,18 +1241,15 @@ int bd_verify_step(const bd_hidden* hidden, const bd_weight* weight, const bd_dr
   DevCtx* ctx = nullptr;
   rc = device_ctx(&ctx);
   if (rc != BD_OK) return rc;
-  BandPlan plan = make_plan(vc.c, ctx->sm_count, ctx->pairs, ctx->quads);
-  VerifyLayout lay = make_verify_layout(vc.c, plan);
-  if (exec && exec->workspace && exec->workspace_bytes < lay.total) {
-    // as fit_layout; then without packed rows, the head decoded in the LM head
-    if (shrink_plan(vc.c, ctx->sm_count, &plan)) lay = make_verify_layout(vc.c, plan);
-    if (exec->workspace_bytes < lay.total && vc.c.split) {
-      if ((rc = check_verify(hidden, weight, draft, eps, variant, &vc, false)) != BD_OK) return rc;
-      plan = make_plan(vc.c, ctx->sm_count, ctx->pairs, ctx->quads);
-      lay = make_verify_layout(vc.c, plan);
-      if (exec->workspace_bytes < lay.total && shrink_plan(vc.c, ctx->sm_count, &plan))
-        lay = make_verify_layout(vc.c, plan);
-    }
+  const size_t ws_bytes = exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX;
+  BandPlan plan;
+  const auto fit = [&] {
+    return fit_call(&vc.c, &plan, ctx->sm_count, ctx->pairs, ctx->quads, ws_bytes, make_verify_layout);
+  };
+  VerifyLayout lay = fit();
+  if (lay.total > ws_bytes && vc.c.split) {  // without packed rows, the head decoded in the LM head
+    if ((rc = check_verify(hidden, weight, draft, eps, variant, &vc, false)) != BD_OK) return rc;
+    lay = fit();
   }
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {
