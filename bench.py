@@ -830,10 +830,17 @@ def e2e_leg(r, K, W, pg, dev):
     return out
 
 
+def restrict_to_single_pairs(world):
+    """Ranks of a job on several GPUs run the LM head without multicast loads, which are for single-GPU runs."""
+    if world > 1:
+        os.environ["BD_PAIR_MC"] = "1"
+
+
 def run_ours(args):
     import paper_2609_33887_gb300 as bdc
 
     rank, world, local = dist_env()
+    restrict_to_single_pairs(world)
     if not torch.cuda.is_available():
         raise SystemExit("bench.py needs a CUDA device (no CPU fallback)")
     torch.cuda.set_device(local)

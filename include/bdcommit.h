@@ -274,7 +274,10 @@ int bd_plan_header(const bd_hidden* hidden, const bd_weight* weight, const bd_ma
  *                        head the kernel decodes itself, else 8192)
  *   BD_PAIR_MC=1|2       single CTA pairs, or clusters of two pairs sharing each
  *                        head tile by multicast (default: clusters for windows of
- *                        at most 512 positions or more than 256 MiB of packed rows)
+ *                        at most 512 positions or more than 256 MiB of packed rows).
+ *                        Multicast loads are for runs on one GPU, over that GPU's
+ *                        own memory: set 1 in every process of a job on several
+ *                        GPUs (bd_lmhead_partials takes single pairs by itself)
  *   BD_PAIR_SHARE=0|1    the two pairs of a cluster share head tiles (two token
  *                        groups, one v-tile at a time) or token rows (one token
  *                        group, two v-tiles at a time); default: head tiles, or

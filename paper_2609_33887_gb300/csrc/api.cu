@@ -93,6 +93,7 @@ struct Call {
   bool either = false;   // a head both the pair kernel (fused) and the one-CTA kernel (a copy) may take
   bool fp8_act = false;  // W8A8: token rows quantised to E4M3, kind::f8f6f4 MMAs on the E4M3 head
   bool verify = false;   // verification rows (bd_verify_step)
+  bool shard = false;    // one rank's shard of the head (bd_lmhead_partials)
   bool split = false;    // W8A16 on the 8-bit path: bf16 rows as two E4M3 terms times the E4M3 head
 };
 
@@ -289,10 +290,12 @@ BandPlan make_plan(const Call& c, int sm_count, int pairs, int quads) {
     // single pairs on all SMs (clusters of 4 leave 8 of 152 SMs idle): windows
     // of at most two token groups, and windows whose packed rows exceed
     // 256 MiB (several bands: the head's L2 and DRAM re-reads dominate).
-    // BD_PAIR_MC = 1 or 2 forces the choice.
+    // BD_PAIR_MC = 1 or 2 forces the choice. The clusters' multicast loads are
+    // for single-GPU runs only: a rank of a vocabulary-parallel head takes
+    // single pairs whatever the variable says.
     const int64_t rows_bytes = c.P * row_operand_bytes(c);
     const int mc_auto = (c.P <= 512 || rows_bytes > (int64_t(256) << 20)) ? 2 : 1;
-    if (!c.fused && env_int("BD_PAIR_MC", mc_auto, 1, 2) == 2 && quads > 0) {
+    if (!c.fused && !c.shard && env_int("BD_PAIR_MC", mc_auto, 1, 2) == 2 && quads > 0) {
       p.mc = 2;
       p.G = quads;
       // the cluster's two pairs share head tiles (two token groups, one v-tile
@@ -370,11 +373,19 @@ Layout make_layout(const Call& c, const BandPlan& p) {
 
 // A plan with fewer partial slots, for a workspace that does not hold those of
 // *p (true if it changed): without the device's choice between the cluster
-// layouts, and the SIMT kernel on fewer runners.
-bool shrink_plan(const Call& c, int sm_count, BandPlan* p) {
+// layouts, the SIMT kernel on fewer runners, and a shard's single pairs on the
+// slots that bd_workspace_size, which knows no shards, counts for its head.
+bool shrink_plan(const Call& c, int sm_count, int pairs, int quads, BandPlan* p) {
   const int slots = plan_max_slots(*p);
   p->adapt = 0;
   if (!c.tc) p->G = static_cast<int>(std::min<int64_t>(2 * sm_count, (c.V + 63) / 64));
+  if (c.shard && c.pair) {
+    Call whole = c;
+    whole.shard = false;
+    BandPlan q = make_plan(whole, sm_count, pairs, quads);
+    q.adapt = 0;
+    p->gv_max = std::max(1, plan_max_slots(q) / plan_unit_slots(*p));
+  }
   return plan_max_slots(*p) < slots;
 }
 
@@ -388,7 +399,7 @@ auto fit_call(Call* c, BandPlan* p, int sm_count, int pairs, int quads, size_t b
     -> decltype(layout(*c, *p)) {
   *p = make_plan(*c, sm_count, pairs, quads);
   auto l = layout(*c, *p);
-  if (l.total > bytes && shrink_plan(*c, sm_count, p)) l = layout(*c, *p);
+  if (l.total > bytes && shrink_plan(*c, sm_count, pairs, quads, p)) l = layout(*c, *p);
   if (l.total > bytes && c->either && !c->split && !c->fp8_act) {
     c->pair = c->fused = !c->fused;
     *p = make_plan(*c, sm_count, pairs, quads);
@@ -810,6 +821,7 @@ int bd_lmhead_partials(const bd_hidden* hidden, const bd_weight* shard, int64_t 
   Call c;
   int rc = check_args(hidden, shard, &local, &tg, exec ? exec->variant : 0, &c);
   if (rc != BD_OK) return rc;
+  c.shard = true;
   if (c.P == 0) return BD_OK;
   if (!out->m || !out->s || !out->a) return BD_ERR_NULL;
   if (!aligned(out->m, 4) || !aligned(out->s, 4) || !aligned(out->a, 4)) return BD_ERR_ALIGN;

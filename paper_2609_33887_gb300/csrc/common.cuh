@@ -77,6 +77,7 @@ struct BandPlan {
   int vc;         // v-tiles a runner takes at once (1, or 2 for 4-CTA clusters sharing token rows)
   int adapt;      // 1: clusters with mc = 2 take vc = 2 instead while the rows form a single token group
   int gv_fixed;   // vocabulary parts when > 0 (clamped to 1..min(G, n_vt)), else chosen
+  int gv_max;     // vocabulary parts at most when > 0 (a workspace with fewer partial slots)
   int rr;         // 1: units taken round-robin (runner c: units c, c + G, ...) instead of packed rounds
   int G2;         // spill runners: single CTA pairs on the SMs the clusters leave free (0: none)
   int spill_pct;  // a spill pair's time per tile against a cluster pair's, in percent (0: 100)
@@ -236,8 +237,14 @@ __host__ __device__ __forceinline__ void plan_gm_range(const BandPlan& p, int bm
   if (*hi < 1) *hi = 1;
 }
 
+// The most vocabulary parts of a launch over `steps` steps of v-tiles.
+__host__ __device__ __forceinline__ int plan_max_parts(const BandPlan& p, int steps) {
+  const int top = p.G < steps ? p.G : steps;
+  return p.gv_max > 0 && p.gv_max < top ? p.gv_max : top;
+}
+
 __host__ __device__ __forceinline__ void plan_gv_range(const BandPlan& p, int* lo, int* hi) {
-  const int top = p.G < p.n_vt ? p.G : p.n_vt;
+  const int top = plan_max_parts(p, p.n_vt);
   if (p.gv_fixed > 0) {
     *lo = *hi = p.gv_fixed < top ? p.gv_fixed : top;
   } else {
@@ -394,6 +401,7 @@ __host__ __device__ __forceinline__ BandPlan plan_share(const BandPlan& p, int v
     q.cpu = SPILL_UNIT_SLOTS;
     q.GM = 0;
     q.gv_fixed = 0;
+    q.gv_max = 0;
   }
   return q;
 }
@@ -446,12 +454,10 @@ __host__ __device__ __forceinline__ int hdr_word(const int* hdr, int i) {
 
 // Partial slots per row the arrays hold at most, over both launches.
 __host__ __device__ __forceinline__ int plan_max_slots(const BandPlan& p) {
-  const int steps = cdiv(p.n_vt, plan_vc(p));
-  int s = plan_unit_slots(p) * (p.G < steps ? p.G : steps);
+  int s = plan_unit_slots(p) * plan_max_parts(p, cdiv(p.n_vt, plan_vc(p)));
   if (p.adapt) {  // and as a single token group
     const BandPlan q = plan_resolve(p, 0);
-    const int steps1 = cdiv(q.n_vt, plan_vc(q));
-    const int s1 = plan_unit_slots(q) * (q.G < steps1 ? q.G : steps1);
+    const int s1 = plan_unit_slots(q) * plan_max_parts(q, cdiv(q.n_vt, plan_vc(q)));
     s = s1 > s ? s1 : s;
   }
   if (p.G2 > 0) s += SPILL_UNIT_SLOTS * (p.G2 < p.n_vt ? p.G2 : p.n_vt);

@@ -104,3 +104,14 @@ def test_both_arms_print_the_same_config_object():
     assert a == b
     assert a["workload"] == TINY_F32.name and a["masked_positions_per_rank"] == n
     assert set(a["inputs_sha256"]) >= {"hidden", "weight", "pos_masked", "block_flags"}
+
+
+def test_ranks_of_a_job_on_several_gpus_run_single_pairs(monkeypatch):
+    monkeypatch.delenv("BD_PAIR_MC", raising=False)
+    bench.restrict_to_single_pairs(1)
+    assert "BD_PAIR_MC" not in os.environ  # a run on one GPU keeps the library's choice
+    for before in (None, "2"):
+        if before:
+            monkeypatch.setenv("BD_PAIR_MC", before)
+        bench.restrict_to_single_pairs(2)
+        assert os.environ["BD_PAIR_MC"] == "1"

@@ -112,8 +112,8 @@ def test_split_agrees_with_the_single_call(name):
 @pytest.mark.parametrize("share", ["0", "1"])
 @pytest.mark.parametrize("name", ["bf16_4", "e4m3_3"])
 def test_split_with_spill_pairs(name, share, monkeypatch):
-    # each shard's LM head on clusters of two pairs (sharing head tiles or
-    # token rows) plus the spill launch
+    # clusters of two pairs (sharing head tiles or token rows) and the spill
+    # launch, asked for: each shard's LM head runs single pairs all the same
     monkeypatch.setenv("BD_PAIR_MC", "2")
     monkeypatch.setenv("BD_PAIR_SPILL", "1")
     monkeypatch.setenv("BD_SPILL_PCT", "50")
