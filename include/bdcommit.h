@@ -105,16 +105,18 @@ typedef struct {
  *   ld * element size (bytes for BD_NVFP4) a multiple of 16.
  *   Both quantised formats decode exactly to bf16. A BD_E4M3 head on the
  *   commit step is read as it is by the 8-bit tensor path of the CTA-pair
- *   kernel at every window size (see bd_exec.variant), with no copy; so it is
- *   for verification, whose rows are then packed in the workspace (a caller's
- *   workspace without room for them is taken too, the codes being decoded as
- *   below). For the other cases the CTA-pair kernel decodes the codes itself,
- *   so the workspace holds no bf16 copy of the head, when a row holds at least
- *   16 bytes of codes and, for BD_NVFP4, `block_scale` is 16-byte aligned with
- *   block_ld a multiple of 16; otherwise the head is first decoded into a bf16
- *   copy in the workspace (bd_workspace_size accounts for it). The environment
- *   variables BD_E4M3_SPLIT=0 (no 8-bit path) and BD_FUSED_DECODE=0 (no decode
- *   in the kernel) select the other paths. */
+ *   kernel at every window size (see bd_exec.variant), with no copy. There each
+ *   bf16 row is held as two E4M3 terms: elements of at least 2^-10 of the row's
+ *   largest exactly, smaller ones to within 2^-17 of it (a row with one element
+ *   1000 times the rest: logits off by about 1e-2; an infinite element saturates).
+ *   For the other cases (verification among them, whose rows are multiplied as
+ *   they are) the CTA-pair kernel decodes the codes itself, so the workspace
+ *   holds no bf16 copy of the head, when a row holds at least 16 bytes of codes
+ *   and, for BD_NVFP4, `block_scale` is 16-byte aligned with block_ld a multiple
+ *   of 16; otherwise the head is first decoded into a bf16 copy in the workspace
+ *   (bd_workspace_size accounts for it). The environment variables
+ *   BD_E4M3_SPLIT=0 (no 8-bit path) and BD_FUSED_DECODE=0 (no decode in the
+ *   kernel) select the other paths. */
 typedef struct {
   const void* data;
   int32_t dtype;
@@ -265,7 +267,8 @@ int bd_plan_header(const bd_hidden* hidden, const bd_weight* weight, const bd_ma
 
 /* ------------------------------------------------------------ tuning knobs --
  * Environment variables read at every call (none is needed; each changes how
- * the work is done, never what is computed):
+ * the work is done, never what is computed, but for the rounding that
+ * BD_E4M3_SPLIT=0 avoids, see bd_weight):
  *   BD_E4M3_SPLIT=0      E4M3 heads not on the 8-bit path (see bd_exec.variant)
  *   BD_FUSED_DECODE=0    quantised heads decoded to a bf16 copy, not in the kernel
  *   BD_PAIR_MAX_P=n      the automatic choice takes the CTA-pair kernel for

@@ -184,11 +184,14 @@ int check_head(const bd_hidden* h, const bd_weight* w, int64_t rows, int variant
   return BD_OK;
 }
 
-// An E4M3 head: the pair kernel multiplies its codes directly on the 8-bit
-// tensor path, with the bf16 rows packed as two E4M3 terms (needs 16-byte
-// aligned code rows), at every window size. 64 x (4 + 1) verification rows
-// (d = 3584, V = 152064) take 233 us this way and 412 us with the codes decoded
-// to bf16 in the kernel, whose converter warps bound it.
+// An E4M3 head on the commit step: the pair kernel multiplies its codes
+// directly on the 8-bit tensor path, with the bf16 rows packed as two E4M3
+// terms (needs 16-byte aligned code rows), at every window size. Verification
+// keeps the rows as they are, the codes decoded to bf16 in the kernel: two
+// terms round elements below 2^-10 of their row's largest, which moves the
+// logits of a row with an element 1000 times the rest by 1e-2 and so the
+// lossless bit. 64 x (4 + 1) rows (d = 3584, V = 152064) take 251 us, 228 us as
+// two terms; 5 rows (d = 4096, V = 128256) 103 and 90 us.
 void choose_split(const bd_weight* w, int variant, Call* c) {
   if (c->tc && w->dtype == BD_E4M3 && (variant == 0 || variant == 3) && env_int("BD_E4M3_SPLIT", 1, 0, 1) != 0 &&
       aligned(w->data, 16) && w->ld % 16 == 0 && w->dim >= 16) {
@@ -1098,7 +1101,7 @@ struct VerifyCall {
 };
 
 int check_verify(const bd_hidden* h, const bd_weight* w, const bd_draft* dr, const bd_eps_grid* eg, int variant,
-                 VerifyCall* vc, bool allow_split = true) {
+                 VerifyCall* vc) {
   if (!h || !w || !dr || !eg) return BD_ERR_NULL;
   if (!eg->eps || eg->E < 1 || eg->E > 31) return BD_ERR_TAU;
   for (int k = 0; k < eg->E; ++k)
@@ -1112,7 +1115,6 @@ int check_verify(const bd_hidden* h, const bd_weight* w, const bd_draft* dr, con
   if (const int rc = check_head(h, w, R, variant, &c, true)) return rc;
   if (R > 0 && !dr->draft) return BD_ERR_NULL;
   if (R > 0 && !aligned(dr->draft, 4)) return BD_ERR_ALIGN;
-  if (allow_split) choose_split(w, variant, &c);
   c.P = R;
   c.n_seq = dr->n_req;
   c.n_slots = 1;
@@ -1121,14 +1123,14 @@ int check_verify(const bd_hidden* h, const bd_weight* w, const bd_draft* dr, con
   c.mask_id = -1;  // the target's full distribution
   c.verify = true;
   c.T = eg->E;
-  c.ldc = h->ld;  // the rows are read in place (two E4M3 terms of them with c.split)
+  c.ldc = h->ld;  // the rows are read in place
   vc->n_req = dr->n_req;
   vc->n_draft = dr->n_draft;
   return BD_OK;
 }
 
 struct VerifyLayout {
-  size_t hdr, idx, draft_row, pm, ps, pa, pt, px, hc, tsc, wq, total;
+  size_t hdr, idx, draft_row, pm, ps, pa, pt, px, wq, total;
 };
 
 VerifyLayout make_verify_layout(const Call& c, const BandPlan& p) {
@@ -1150,8 +1152,6 @@ VerifyLayout make_verify_layout(const Call& c, const BandPlan& p) {
   l.pa = take(4 * slots * R, 256);
   l.pt = take(4 * slots * R, 256);
   l.px = take(4 * slots * R, 256);
-  l.hc = c.split ? take(2 * static_cast<size_t>(round_up(c.d, 16)) * R, 1024) : 0;
-  l.tsc = c.split ? take(4 * R, 256) : 0;
   l.wq = decoded_head(c) ? take(2 * static_cast<size_t>(c.ldq) * static_cast<size_t>(c.V), 1024) : 0;
   l.total = (off + 255) / 256 * 256;
   return l;
@@ -1180,18 +1180,11 @@ int run_verify(const VerifyCall& vc, const BandPlan& plan, const VerifyLayout& l
   prep.draft_row = draft_row;
   prep.n_rows = n_rows;
   prep.plan = plan;
-  prep.hidden = static_cast<const __nv_bfloat16*>(hidden->data);
-  prep.ld = c.ldh;
-  prep.d = static_cast<int>(c.d);
-  prep.hc = c.split ? ws + lay.hc : nullptr;
-  prep.ldc = ld_fp8_rows(c);
-  prep.tok_scale = c.split ? reinterpret_cast<float*>(ws + lay.tsc) : nullptr;
-  int rc = cuda_status(bd::launch_prep_verify(prep, c.split ? bd::ROWS_E4M3X2 : bd::ROWS_BF16, st));
+  int rc = cuda_status(bd::launch_prep_verify(prep, st));
   if (rc != BD_OK) return rc;
 
-  rc = launch_lmhead(c, plan, hidden, weight, c.split ? prep.hc : hidden->data, c.split ? prep.ldc : c.ldh,
-                     ws + lay.wq, idx, n_rows, draft_row, Partials{pm, ps, pa, pt, px}, status, sm_count, ev_begin,
-                     ev_end, st, prep.tok_scale);
+  rc = launch_lmhead(c, plan, hidden, weight, hidden->data, c.ldh, ws + lay.wq, idx, n_rows, draft_row,
+                     Partials{pm, ps, pa, pt, px}, status, sm_count, ev_begin, ev_end, st);
   if (rc != BD_OK) return rc;
 
   bd::VerifyArgs va;
@@ -1253,16 +1246,9 @@ int bd_verify_step(const bd_hidden* hidden, const bd_weight* weight, const bd_dr
   DevCtx* ctx = nullptr;
   rc = device_ctx(&ctx);
   if (rc != BD_OK) return rc;
-  const size_t ws_bytes = exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX;
   BandPlan plan;
-  const auto fit = [&] {
-    return fit_call(&vc.c, &plan, ctx->sm_count, ctx->pairs, ctx->quads, ws_bytes, make_verify_layout);
-  };
-  VerifyLayout lay = fit();
-  if (lay.total > ws_bytes && vc.c.split) {  // without packed rows, the head decoded in the LM head
-    if ((rc = check_verify(hidden, weight, draft, eps, variant, &vc, false)) != BD_OK) return rc;
-    lay = fit();
-  }
+  const VerifyLayout lay = fit_call(&vc.c, &plan, ctx->sm_count, ctx->pairs, ctx->quads,
+                                    exec && exec->workspace ? exec->workspace_bytes : SIZE_MAX, make_verify_layout);
   uint8_t* ws = nullptr;
   if (exec && exec->workspace) {
     if (exec->workspace_bytes < lay.total) return BD_ERR_WORKSPACE;

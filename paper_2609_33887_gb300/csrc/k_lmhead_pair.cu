@@ -253,8 +253,6 @@ static_assert(stage_count<HF_W8A8, false>(160) == 7 && stage_count<HF_W8A8, fals
               "W8A8: seven 26 KB stages at NT = 160, five 32 KB stages at NT = 256");
 static_assert(stage_count<HF_E4M3X2, false>(160) == 5 && stage_count<HF_E4M3X2, false>(256) == 4,
               "two-term rows: five 36 KB stages at NT = 160, four 48 KB stages at NT = 256");
-static_assert(stage_count<HF_E4M3X2, true>(160) == 5 && stage_count<HF_E4M3X2, true>(256) == 4,
-              "two-term rows: the same stages on the verification path");
 // Sets of converter warps that take operand stages in turn. A barrier's parity
 // tells two neighbouring uses of a stage apart, so a set that comes to stage g
 // must know that use g - 2 NS of that operand stage is over, and that the raw
@@ -332,7 +330,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   constexpr int MAX_CHUNKS = max_chunks<HF>();
   constexpr bool W8A8 = HF == HF_W8A8;
   constexpr bool X2 = HF == HF_E4M3X2;
-  static_assert(!(W8A8 && VERIFY), "W8A8 serves the commit step");
+  static_assert(!((W8A8 || X2) && VERIFY), "the 8-bit instantiations serve the commit step");
   // commit step with a head decoded in the kernel: f16 operands (the decode
   // ends at f16), token rows pre-scaled by a power of two per row
   constexpr bool F16OPS = QUANT && !VERIFY;
@@ -801,7 +799,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
                   s[c] = 0.f;
                   t[c] = 0.f;
                 } else {
-                  const float dm = (m[c] - cm) * k2[c];
+                  const float dm = (m[c] - cm) * LOG2E;
                   const float f = ex2_approx(dm);
                   t[c] = f * fmaf(dm, s[c], t[c]);
                   s[c] *= f;
@@ -873,7 +871,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
           st(ew, ST_A)[c * 32 + lane] = __int_as_float(arg[c]);
           if constexpr (VERIFY) {
             st(ew, ST_T)[c * 32 + lane] = t[c];
-            st(ew, ST_X)[c * 32 + lane] = TOKS ? lx[c] * ts[c] : lx[c];
+            st(ew, ST_X)[c * 32 + lane] = lx[c];
           }
         }
       }
@@ -1044,9 +1042,8 @@ cudaError_t launch_lmhead_pair(const PairTokenMaps& tmH, const CUtensorMap& tmW,
       if (verify) return cudaErrorInvalidValue;
       return launch_pair<HF_W8A8, false>(tmH, tmW, q, lo, a, st);
     case HF_E4M3X2:
-      if (tmLo == nullptr) return cudaErrorInvalidValue;
-      return verify ? launch_pair<HF_E4M3X2, true>(tmH, tmW, q, lo, a, st)
-                    : launch_pair<HF_E4M3X2, false>(tmH, tmW, q, lo, a, st);
+      if (verify || tmLo == nullptr) return cudaErrorInvalidValue;
+      return launch_pair<HF_E4M3X2, false>(tmH, tmW, q, lo, a, st);
     case HF_E4M3:
       return verify ? launch_pair<HF_E4M3, true>(tmH, tmW, q, lo, a, st)
                     : launch_pair<HF_E4M3, false>(tmH, tmW, q, lo, a, st);

@@ -388,14 +388,11 @@ cudaError_t launch_prep_rows(const PrepArgs& args, int row_format, int sm_count,
 }
 
 // ---------------------------------------------------------------------------
-// Verification rows need no compaction: every row is live. Row
-// r = q * (n_draft + 1) + i verifies draft token i of request q (i < n_draft);
-// the last row of a request verifies nothing. bf16 and NVFP4 heads read the
-// caller's rows in place (ROWS_BF16 here: nothing to pack); an E4M3 head on
-// the 8-bit path reads them as two E4M3 terms, packed by one warp per row.
+// Verification rows need no compaction: every row is live, and the LM head
+// reads the caller's rows in place. Row r = q * (n_draft + 1) + i verifies draft
+// token i of request q (i < n_draft); the last row of a request verifies nothing.
 // ---------------------------------------------------------------------------
-template <int FMT, int RC>
-__global__ void __launch_bounds__(PREP_THREADS, 2) prep_verify_kernel(PrepVerifyArgs a) {
+__global__ void __launch_bounds__(PREP_THREADS) prep_verify_kernel(PrepVerifyArgs a) {
   __shared__ PlanScratch plan_s;
   griddep_launch_dependents();
   griddep_wait();
@@ -404,33 +401,19 @@ __global__ void __launch_bounds__(PREP_THREADS, 2) prep_verify_kernel(PrepVerify
     plan_write_header(a.plan, R, a.n_rows, &plan_s);
     return;
   }
-  const int cta = static_cast<int>(blockIdx.x) - 1, ctas = static_cast<int>(gridDim.x) - 1;
-  for (int r = cta * PREP_THREADS + threadIdx.x; r < R; r += ctas * PREP_THREADS) {
+  for (int r = (blockIdx.x - 1) * PREP_THREADS + threadIdx.x; r < R; r += (gridDim.x - 1) * PREP_THREADS) {
     const int q = r / (D + 1), i = r % (D + 1);
     a.idx[r] = r;
     a.draft_row[r] = i < D ? a.draft[q * D + i] : -1;
   }
-  if constexpr (FMT != ROWS_BF16) {
-    const int64_t row_bytes = packed_row_bytes<FMT>(a.ldc);
-    for (int r = cta * PREP_WARPS + static_cast<int>(threadIdx.x >> 5); r < R; r += ctas * PREP_WARPS) {
-      const float scale = pack_row<FMT, RC>(a.hidden + static_cast<int64_t>(r) * a.ld, a.d,
-                                            static_cast<uint8_t*>(a.hc) + r * row_bytes, R * row_bytes);
-      if ((threadIdx.x & 31) == 0) a.tok_scale[r] = scale;
-    }
-  }
 }
 
-cudaError_t launch_prep_verify(const PrepVerifyArgs& a, int row_format, cudaStream_t st) {
-  if (row_format != ROWS_BF16 && row_format != ROWS_E4M3X2) return cudaErrorInvalidValue;
+cudaError_t launch_prep_verify(const PrepVerifyArgs& a, cudaStream_t st) {
   const int R = a.n_req * (a.n_draft + 1);
-  const int rows = row_format == ROWS_BF16 ? PREP_THREADS : PREP_WARPS;  // per CTA
-  int grid = (R + rows - 1) / rows;
+  int grid = (R + PREP_THREADS - 1) / PREP_THREADS;
   if (grid < 1) grid = 1;
   if (grid > 1024) grid = 1024;
-  auto* kern = row_format == ROWS_BF16 ? prep_verify_kernel<ROWS_BF16, 1>
-               : a.d <= 2048           ? prep_verify_kernel<ROWS_E4M3X2, 8>
-                                       : prep_verify_kernel<ROWS_E4M3X2, 20>;
-  return launch_behind(kern, 1 + grid, st, a);
+  return launch_behind(prep_verify_kernel, 1 + grid, st, a);
 }
 
 // ---------------------------------------------------------------------------

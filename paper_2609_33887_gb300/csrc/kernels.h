@@ -187,8 +187,7 @@ cudaError_t launch_merge_commit(const CommitArgs& a, cudaStream_t st, int mode =
 // token draft[q * n_draft + i], the last row of a request gives its bonus token.
 // Prep: idx[r] = r, draft_row[r] = that draft token or -1, and the workspace
 // header n_rows (R and the LM head's plan for R rows, HDR_* words of
-// common.cuh); with ROWS_E4M3X2 also the rows as two E4M3 terms in hc (as
-// launch_prep_rows), with ROWS_BF16 the LM head reads them in place.
+// common.cuh). The LM head reads the caller's rows in place.
 struct PrepVerifyArgs {
   const int32_t* draft;
   int n_req, n_draft;
@@ -196,14 +195,8 @@ struct PrepVerifyArgs {
   int* draft_row;
   int* n_rows;
   BandPlan plan;
-  const __nv_bfloat16* hidden;
-  int64_t ld;
-  int d;
-  void* hc;
-  int64_t ldc;
-  float* tok_scale;
 };
-cudaError_t launch_prep_verify(const PrepVerifyArgs& a, int row_format, cudaStream_t st);
+cudaError_t launch_prep_verify(const PrepVerifyArgs& a, cudaStream_t st);
 
 struct VerifyArgs {
   const int* draft_row;

@@ -131,8 +131,8 @@ def test_verify_step(head, V, n_req):
 
 
 def test_verify_with_the_workspace_of_rows_read_in_place(monkeypatch):
-    # an E4M3 head's rows are packed in the workspace; one that has no room for
-    # them is taken as well (the head is then decoded in the kernel)
+    # verification on an E4M3 head reads its rows in place (the head is decoded
+    # in the kernel), whatever room there is beyond the partial slots
     n_req, D, d, V = 6, 4, 336, 700
     h, w, scale, logit = make("e4m3", n_req * (D + 1), V, d, 3)
     draft = logit.argmax(1).view(n_req, D + 1)[:, :D].int().reshape(-1).contiguous()
@@ -149,8 +149,8 @@ def test_verify_with_the_workspace_of_rows_read_in_place(monkeypatch):
 
 
 def test_verify_with_the_workspace_of_a_decoded_copy(monkeypatch):
-    # more rows than vocabulary entries: the packed rows need more room than
-    # the head's bf16 copy, beside which only the slots of shared head tiles fit
+    # the head decoded to a bf16 copy, with room beside it for the slots of
+    # shared head tiles only
     n_req, D, d, V = 60, 4, 336, 200
     h, w, scale, logit = make("e4m3", n_req * (D + 1), V, d, 5)
     draft = logit.argmax(1).view(n_req, D + 1)[:, :D].int().reshape(-1).contiguous()
