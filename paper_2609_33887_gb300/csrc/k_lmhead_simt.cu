@@ -23,6 +23,7 @@
 // wider tile, with more, smaller stages in flight (32 rows, d = 256, V = 4096:
 // 17 us, latency). The host chooses C (simt_tile).
 #include <atomic>
+#include <cfloat>
 #include <cuda_fp16.h>
 
 #include "bdcommit.h"
@@ -47,6 +48,13 @@ __host__ __device__ constexpr int ctas_of() { return VERIFY ? SIMT_CTAS_VERIFY :
 __device__ __forceinline__ float load_h(const void* p, int64_t i, int dt) {
   if (dt == BD_F32) return static_cast<const float*>(p)[i];
   return __bfloat162float(static_cast<const __nv_bfloat16*>(p)[i]);
+}
+
+// The smaller of two, NaN if either is.
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float d;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
 }
 
 __device__ __forceinline__ float e4m3_to_float(uint8_t c) {
@@ -243,9 +251,12 @@ __device__ __forceinline__ void run_unit(const SimtArgs& a, SimtSmem<C, VERIFY>&
         m = cm;
       }
       if (m != -INFINITY) {
+        // an infinite maximum (logits that overflowed) counts 1 like any other:
+        // u is cut at 0, against the largest finite number; NaN stays NaN
+        const float base = fminf(m, FLT_MAX);
 #pragma unroll
         for (int j = 0; j < C; ++j) {
-          const float u = (x[j] - m) * LOG2E;
+          const float u = min_nan((x[j] - base) * LOG2E, 0.f);
           const float e = ex2_approx(u);
           s += e;
           // -inf logits give e = 0; clamping u keeps e * u at 0

@@ -115,3 +115,35 @@ def test_scratch_that_holds_fewer_partials():
     tok, conf, commit, _ = bdc.commit_step(h, w, ones, ones, N, 1, 1, [0.5])
     torch.cuda.synchronize()
     assert torch.equal(out[0], tok) and float((out[1] - conf).abs().max()) < 1e-5
+
+
+@pytest.mark.parametrize("V", [300, 5000, 9000, 40000])  # tiles of 32, 64, 112 and 128 entries
+@pytest.mark.parametrize("N", [1, 40, 77])
+def test_infinite_and_missing_logits(N, V):
+    # a head row that overflows to one infinite logit takes all the probability
+    # (two such rows half each, the lower id), one of -inf takes none, and a NaN
+    # logit leaves no confidence: nothing commits without the fallback
+    d = 16
+    g = torch.Generator(device="cuda").manual_seed(V + N)
+    h, w = torch.randn(N, d, generator=g, device="cuda"), torch.randn(V, d, generator=g, device="cuda")
+    ones = torch.ones(N, dtype=torch.uint8, device="cuda")
+    step = lambda h, w: bdc.commit_step(h, w, ones, ones, N, 1, 1, [0.25])  # noqa: E731
+    h[:, 0], w[:, 0] = 1e30, 0.0
+    top = (V * 2 // 3, V - 1)
+    for n in (1, 2):
+        w[top[-n:], 0] = 1e30  # 1e60: infinite in float32
+        tok, conf, commit, _ = step(h, w)
+        assert torch.equal(tok, torch.full_like(tok, top[-n])) and torch.equal(conf, torch.full_like(conf, 1 / n))
+        assert torch.equal(commit, torch.ones_like(commit))
+    w[top[0], 0] = w[top[1], 0] = -1e30
+    tok, conf, _, _ = step(h, w)
+    live = torch.ones(V, dtype=torch.bool, device="cuda")
+    live[list(top)] = False
+    assert live[tok.long()].all()
+    logit = h[:, 1:].double() @ w[:, 1:].double().t()
+    p = (logit[:, live].amax(1) - logit[:, live].logsumexp(1)).exp()
+    assert float((conf.double() - p).abs().max()) < TOL
+    w[V // 4, 3] = float("nan")
+    _, conf, commit, _ = step(h, w)
+    assert torch.isnan(conf).all() and not commit.any()
+    assert bdc.bd_get_device_status() == 0
