@@ -260,9 +260,9 @@ int64_t head_operand_bytes(const Call& c) {
 // groups (of 96) the window may hold: 32 entries up to a tile per SM (per
 // runner for verification), 64 up to 1.5 per SM (not for verification, which
 // has two CTAs per SM). LM head, float32, 128 / 112 / 64 / 32 entries: 15 rows,
-// d = 256, V = 4096 19.5 / 19.5 / 19.5 / 16.4 us; d = 512, 75 rows, V = 5000
-// 47 / 45 / 39 / 53, V = 12000 60 / 54 / 47 / 76, V = 20000 70 / 68 / 93 / 131,
-// 250 rows, V = 12000 100 / 93 / 111 / 228. Verification, 15 rows, V = 5000
+// d = 256, V = 4096 19.4 / 19.1 / 19.4 / 16.4 us; d = 512, 75 rows, V = 5000
+// 46 / 44 / 39 / 45, V = 12000 59 / 53 / 47 / 70, V = 20000 70 / 68 / 92 / 108,
+// 250 rows, V = 12000 100 / 92 / 110 / 145. Verification, 15 rows, V = 5000
 // 29 / 28 / 28 / 24, 75 rows, V = 12000 53 / 55 / 66 / 72. Of the wide ones the
 // width whose tiles on the SM with most of them are fewer entries, summed over
 // the groups the window may come to: V = 50304, 75 rows 117 / 107, 500 rows
@@ -270,7 +270,7 @@ int64_t head_operand_bytes(const Call& c) {
 int simt_tile(const Call& c, int sm_count) {
   const int64_t groups = std::min<int64_t>((c.P + 95) / 96, 8), half = ((c.P + 95) / 96 + 1) / 2;
   const auto tiles = [&c](int64_t g, int bn) { return g * ((c.V + bn - 1) / bn); };
-  if (tiles(half, 32) <= (c.verify ? bd::SIMT_CTAS_VERIFY : 1) * sm_count) return 32;
+  if (tiles(half, 32) <= (c.verify ? bd::simt_ctas(32, true) : 1) * sm_count) return 32;
   if (!c.verify && 2 * tiles(half, 64) <= 3 * sm_count) return 64;
   int64_t narrow = 0, wide = 0;
   for (int64_t g = 1; g <= groups; ++g) {
@@ -330,8 +330,8 @@ BandPlan make_plan(const Call& c, int sm_count, int pairs, int quads) {
     p.cpu = 1;
   } else {
     p.BM = bd::BM_SIMT;
-    p.G = (c.verify ? bd::SIMT_CTAS_VERIFY : bd::SIMT_CTAS) * sm_count;
     p.BN = simt_tile(c, sm_count);
+    p.G = bd::simt_ctas(p.BN, c.verify) * sm_count;
     p.cpu = 1;
   }
   // bands: GM derived on the device from the head and row bytes (0), or fixed

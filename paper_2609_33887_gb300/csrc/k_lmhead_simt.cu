@@ -37,13 +37,13 @@ constexpr int KC = 16;      // columns of d per stage
 constexpr int KS = KC + 4;  // row stride of a stage
 constexpr int THREADS = 128;
 constexpr int MAX_R = 12;
+// shared memory of an SM, and what the system keeps of it per CTA
+constexpr size_t SMEM_PER_SM = 228 * 1024, SMEM_RESERVED = 1024;
 
 template <int C>
 __host__ __device__ constexpr int bn_of() { return 16 * C; }  // entries per tile
 template <int C>
 __host__ __device__ constexpr int stages_of() { return C > 4 ? 3 : C == 4 ? 4 : 6; }
-template <bool VERIFY>
-__host__ __device__ constexpr int ctas_of() { return VERIFY ? SIMT_CTAS_VERIFY : SIMT_CTAS; }
 
 __device__ __forceinline__ float load_h(const void* p, int64_t i, int dt) {
   if (dt == BD_F32) return static_cast<const float*>(p)[i];
@@ -274,7 +274,9 @@ __device__ __forceinline__ void run_unit(const SimtArgs& a, SimtSmem<C, VERIFY>&
 }  // namespace
 
 template <int C, bool VERIFY>
-__global__ void __launch_bounds__(THREADS, ctas_of<VERIFY>()) lmhead_simt_kernel(SimtArgs a) {
+__global__ void __launch_bounds__(THREADS, simt_ctas(bn_of<C>(), VERIFY)) lmhead_simt_kernel(SimtArgs a) {
+  static_assert(simt_ctas(bn_of<C>(), VERIFY) * (sizeof(SimtSmem<C, VERIFY>) + SMEM_RESERVED) <= SMEM_PER_SM,
+                "the CTAs the plan counts on fit an SM");
   extern __shared__ __align__(16) uint8_t smem_raw[];
   SimtSmem<C, VERIFY>& sm = *reinterpret_cast<SimtSmem<C, VERIFY>*>(smem_raw);
   const int tid = threadIdx.x;

@@ -145,9 +145,14 @@ struct SimtArgs {
   float* part_t = nullptr;
   float* part_x = nullptr;
 };
-// CTAs per SM (plan.G = this times the SMs; plan.BM = BM_SIMT; plan.BN = the
-// vocabulary entries per tile: 32, 112 or 128, or 64 outside verification)
-constexpr int SIMT_CTAS = 3, SIMT_CTAS_VERIFY = 2;
+// CTAs per SM, by the vocabulary entries per tile (plan.BN: 32, 112 or 128, or 64
+// outside verification); plan.G = this times the SMs, plan.BM = BM_SIMT. Two with
+// tiles of 32 entries, whose ring of six stages fills an SM with that: a plan for
+// three took more row groups than there were CTAs for (V = 4096, d = 1024, LM
+// head, three / two: 48 rows 67 / 39 us, 77 rows 81 / 50, 192 rows 123 / 80; V =
+// 2500, 96 rows 74 / 45). Four stages, so that three fit, measured as two on
+// several row groups and slower on one (V = 4096, 15 rows 37 / 33 us).
+constexpr int simt_ctas(int bn, bool verify) { return verify || bn == 32 ? 2 : 3; }
 cudaError_t launch_lmhead_simt(const SimtArgs& a, cudaStream_t st);
 
 // a3+a4: merge of the partials per row, then the threshold commit with the

@@ -147,3 +147,17 @@ def test_infinite_and_missing_logits(N, V):
     _, conf, commit, _ = step(h, w)
     assert torch.isnan(conf).all() and not commit.any()
     assert bdc.bd_get_device_status() == 0
+
+
+@pytest.mark.parametrize("V", [2500, 4096, 4800])
+def test_units_of_narrow_tiles_run_at_once(V):
+    # two CTAs with tiles of 32 entries fit an SM: the plan of a window that one
+    # round could hold does not count on more (which staged the head once more
+    # per group and left a second, partial round)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for P in (48, 77, 96, 150, 192):
+        h, w = torch.zeros(P, 64, device="cuda"), torch.zeros(V, 64, device="cuda")
+        ones = torch.ones(P, dtype=torch.uint8, device="cuda")
+        hdr = bdc.bdcommit.bd_plan_header(h, w, None, ones, ones, P, 1, 1, -1, [0.5], P)
+        band, parts = hdr[2], hdr[3]
+        assert band * parts <= 2 * sms
