@@ -114,16 +114,17 @@ __host__ __device__ __forceinline__ int pair_group_rows(int n_rows, int most = 2
 // Rows per group of the SIMT kernel, at most 96, equal sizes rounded up to a
 // multiple of 8 (of 16 above 64). Up to 64 groups, of the four fewest group
 // counts the one whose rounds of tiles times rows cost least, the fewer groups
-// on a tie (77 rows: one group of 80, LM head 223 us against 240 us as two of
-// 40; 256 rows: four of 64, 684 us against 801 us as three of 96).
+// on a tie; the fewest groups beyond.
 __host__ __device__ __forceinline__ int simt_group_rows(const BandPlan& p, int n_rows) {
   if (n_rows <= 0) return 8;
   const int g0 = cdiv(n_rows, 96);
   int best = 0, best_cost = 0;
-  for (int g = g0; g < (g0 <= 64 ? g0 + 4 : g0 + 1); ++g) {
+  for (int g = g0; g < g0 + 4; ++g) {
     int rows = cdiv(n_rows, g);
     rows = rows <= 64 ? cdiv(rows, 8) * 8 : cdiv(rows, 16) * 16;
-    const int cost = cdiv(g * p.n_vt, p.G) * rows;  // 32 bits: g <= 67, n_vt <= 2^23
+    if (g0 > 64) return rows;
+    // 32 bits: g <= 67, n_vt < 2^24 (2^30 entries in tiles of 112), and G is in the hundreds there
+    const int cost = cdiv(g * p.n_vt, p.G) * rows;
     if (best == 0 || cost < best_cost) {
       best = rows;
       best_cost = cost;
@@ -191,7 +192,7 @@ __host__ __device__ __forceinline__ Packing plan_pack(int n_mt, int G, int gm, i
   k.rem = n_mt - k.nb * gm;
   k.k1 = G / gm;
   k.kr = k.rem > 0 ? G / k.rem : 0;
-  // nb * gv < 2^28 (at most 2^19 m-tiles of 2^24 positions, gv <= 304): 32-bit
+  // nb * gv < 2^28 (at most 2^19 m-tiles of 2^24 positions, gv <= 456): 32-bit
   const int full_parts = k.nb * gv;
   k.R0 = full_parts / k.k1;
   k.u0 = (full_parts - k.R0 * k.k1) * gm;
