@@ -376,16 +376,22 @@ Layout make_layout(const Call& c, const BandPlan& p) {
 
 // A plan with fewer partial slots, for a workspace that does not hold those of
 // *p (true if it changed): without the device's choice between the cluster
-// layouts, the SIMT kernel on fewer runners, and a shard's single pairs on the
-// slots that bd_workspace_size, which knows no shards, counts for its head.
+// layouts, the SIMT kernel on fewer runners, and a shard or a W8A8 step, whose
+// layouts bd_workspace_size does not know, on the slots that it counts for the
+// plain step (W8A8 rows of half the bytes take single pairs on windows where
+// two-term rows take clusters).
 bool shrink_plan(const Call& c, int sm_count, int pairs, int quads, BandPlan* p) {
   const int slots = plan_max_slots(*p);
   p->adapt = 0;
   if (!c.tc) p->G = static_cast<int>(std::min<int64_t>(2 * sm_count, (c.V + 63) / 64));
-  if (c.shard && c.pair) {
-    Call whole = c;
-    whole.shard = false;
-    BandPlan q = make_plan(whole, sm_count, pairs, quads);
+  if (c.pair && (c.shard || c.fp8_act)) {
+    Call plain = c;
+    plain.shard = false;
+    if (c.fp8_act) {
+      plain.fp8_act = false;
+      plain.split = true;
+    }
+    BandPlan q = make_plan(plain, sm_count, pairs, quads);
     q.adapt = 0;
     p->gv_max = std::max(1, plan_max_slots(q) / plan_unit_slots(*p));
   }

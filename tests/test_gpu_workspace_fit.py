@@ -98,3 +98,26 @@ def test_verify_step(V, monkeypatch):
         assert bdc.bd_get_device_status() == 0
         rows = torch.arange(0, R, D + 1, device="cuda")
         check(out["tokens"][rows], out["p_draft"][rows], (p[rows], a[rows], gap[rows]))
+
+
+def test_w8a8_in_the_documented_workspace():
+    # bd_workspace_size covers W8A8 too: above 256 MiB of two-term rows the plain
+    # step takes clusters, W8A8 rows of half the bytes single pairs with more partials
+    P, V, d, N = 131100, 40000, 1024, 300
+    g = torch.Generator(device="cuda").manual_seed(3)
+    h = torch.randn(P, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    w = torch.randn(V, d, generator=g, device="cuda") / d ** 0.5
+    scale = w.abs().amax(1) / 448
+    w = (w / scale[:, None]).to(torch.float8_e4m3fn)
+    mask = torch.zeros(P, dtype=torch.uint8, device="cuda")
+    mask[torch.randperm(P, generator=g, device="cuda")[:N]] = 1
+    flags = torch.ones(P, dtype=torch.uint8, device="cuda")
+    args = (h, w, scale, mask, flags, P, 1, 1, -1, [0.5])
+    outs = []
+    for ws in (None, aligned(bdc.bd_workspace_size(*args))):
+        out = [torch.empty(P, dtype=t, device="cuda") for t in (torch.int32, torch.float32, torch.int32)]
+        assert B.bd_commit_step_ex(*args, *out, workspace=ws, flags=B.BD_EXEC_FP8_ACTIVATIONS) == 0
+        assert bdc.bd_get_device_status() == 0
+        outs.append(out)
+    assert torch.equal(outs[0][0], outs[1][0]) and int((outs[0][0] >= 0).sum()) == N
+    assert float((outs[0][1] - outs[1][1]).abs().max()) < 1e-5  # the same float32 sums, grouped by fewer parts
