@@ -24,7 +24,7 @@
 // live in TMEM: three of 160 columns for groups of at most 160 tokens (the
 // epilogue of one tile overlaps two tiles of MMAs), else two of 256.
 //
-// Two pairs per cluster (MC = 2, clusters of 4 CTAs): the pairs
+// Two pairs per cluster (clusters of 4 CTAs): the pairs
 // hold adjacent token groups of the same vocabulary part, so they need the
 // same head tiles. Each head tile is then read from L2 once for both: every
 // CTA loads a 64-row half of its 128 head rows and multicasts it to the CTA
@@ -317,11 +317,12 @@ __device__ __forceinline__ void decode_row(uint32_t raw_base, int h, int row, in
 
 }  // namespace
 
-// MC: CTA pairs per cluster. Only MC = 2 issues multicast loads. They write to
-// shared memory of this GPU's own CTAs, the tensor maps must cover this GPU's
-// memory alone, and only calls of a single-GPU run may take it: a rank of a
-// job on several GPUs runs MC = 1, which holds none.
-template <int HF, bool VERIFY, int MC>
+// MULTICAST: clusters of two CTA pairs (and the spill launch beside them), whose
+// loads are multicast. They write to shared memory of this GPU's own CTAs, the
+// tensor maps must cover this GPU's memory alone, and only calls of a single-GPU
+// run may take it: a rank of a job on several GPUs runs single pairs of the
+// other instantiation, which holds no multicast load.
+template <int HF, bool VERIFY, bool MULTICAST>
 __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     lmhead_pair_kernel(const __grid_constant__ PairTokenMaps tmH, const __grid_constant__ CUtensorMap tmW,
                        const __grid_constant__ PairQuantMaps tmQ, const __grid_constant__ PairTokenMaps tmL,
@@ -342,8 +343,9 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   PairCtl* ctl = reinterpret_cast<PairCtl*>(smem + CTL_OFFSET);
   const uint32_t smem_base = smem_u32(smem);
 
-  // two pairs per cluster share head tiles (mc = 2) or token rows (vc = 2)
-  static_assert(MC == 1 || (MC == 2 && !QUANT), "heads decoded in the kernel run single pairs");
+  static_assert(!(MULTICAST && QUANT), "heads decoded in the kernel run single pairs");
+  // pairs per cluster: two sharing head tiles (mc = 2) or token rows (vc = 2)
+  const int MC = MULTICAST ? plan_mc(a.plan) * plan_vc(a.plan) : 1;
   // launched without its cluster there is no peer CTA to map or to pair
   // MMAs with: report and do nothing
   if (cluster_nctarank() != static_cast<uint32_t>(2 * MC)) {
@@ -404,7 +406,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   if (!spill) griddep_wait();
   if (!spill && a.plan.G2 > 0) griddep_launch_dependents();
   const int n_rows = static_cast<int>(warp_uniform(static_cast<uint32_t>(hdr_word(a.n_rows, HDR_N))));
-  const int VC = MC == 1 ? 1 : plan_vc(plan_resolve(a.plan, n_rows));
+  const int VC = MULTICAST ? plan_vc(plan_resolve(a.plan, n_rows)) : 1;
   const int pp_mt = VC == 1 ? pp : 0;  // this pair's token group within the runner's m-tiles
   constexpr int BK = STAGE_K;
   constexpr int ACOLS = atom_cols<HF>();
@@ -475,22 +477,22 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
                 if (MC == 1 || VC == 2) {
                   tma_load_2d_pair(sa + j * A_BLOCK, &tmW, fb, kb * BK + ACOLS * j, vrow, pol_w);
                   tma_load_2d_pair(sa + j * A_BLOCK + A_BLOCK / 2, &tmW, fb, kb * BK + ACOLS * j, vrow + 64, pol_w);
-                } else if constexpr (MC == 2) {
+                } else if constexpr (MULTICAST) {
                   tma_load_2d_pair_mc(sa + j * A_BLOCK + pp * (A_BLOCK / 2), &tmW, fb, kb * BK + ACOLS * j,
                                       vrow + 64 * pp, head_mc, pol_w);
                 }
                 // this CTA's token rows, or its quarter of the rows both pairs share
-                if (MC == 1 || VC == 1) {
+                if (!MULTICAST || VC == 1) {
                   tma_load_2d_pair(sa + NATOM * A_BLOCK + j * B_BLOCK, tm_tok, fb, kb * BK + ACOLS * j, tok0, pol_h);
-                } else if constexpr (MC == 2) {
+                } else if constexpr (MULTICAST) {
                   tma_load_2d_pair_mc(sa + NATOM * A_BLOCK + j * B_BLOCK + pp * (B_BLOCK / 2), tm_tok_q, fb,
                                       kb * BK + ACOLS * j, tok0 + pp * (half / 2), head_mc, pol_h);
                 }
               }
               if constexpr (X2) {
-                if (MC == 1 || VC == 1) {
+                if (!MULTICAST || VC == 1) {
                   tma_load_2d_pair(sa + A_BLOCK + B_BLOCK, tm_lo, fb, kb * BK, tok0, pol_h);
-                } else if constexpr (MC == 2) {
+                } else if constexpr (MULTICAST) {
                   tma_load_2d_pair_mc(sa + A_BLOCK + B_BLOCK + pp * (B_BLOCK / 2), tm_lo_q, fb, kb * BK,
                                       tok0 + pp * (half / 2), head_mc, pol_h);
                 }
@@ -932,7 +934,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
 
 size_t pair_smem_bytes() { return SMEM_BYTES; }
 
-template <int HF, bool VERIFY, int MC>
+template <int HF, bool VERIFY, bool MULTICAST>
 static cudaError_t pair_opt_in() {
   static std::atomic<uint64_t> opted_in{0};
   int dev = 0;
@@ -940,7 +942,7 @@ static cudaError_t pair_opt_in() {
   if (e != cudaSuccess) return e;
   const uint64_t bit = 1ull << (dev & 63);
   if ((opted_in.load() & bit) == 0) {
-    e = cudaFuncSetAttribute(lmhead_pair_kernel<HF, VERIFY, MC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(lmhead_pair_kernel<HF, VERIFY, MULTICAST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(SMEM_BYTES));
     if (e != cudaSuccess) return e;
     opted_in.fetch_or(bit);
@@ -970,58 +972,59 @@ static void pair_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int 
   }
 }
 
-template <int MC>
-static cudaError_t max_clusters(int sm_count, int* clusters) {
-  cudaError_t e = pair_opt_in<HF_BF16, false, MC>();
+template <bool MULTICAST>
+static cudaError_t max_clusters(int sm_count, int mc, int* clusters) {
+  cudaError_t e = pair_opt_in<HF_BF16, false, MULTICAST>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  pair_config(&cfg, attr, sm_count / (2 * MC), pair_threads<HF_BF16>(), nullptr, false, MC);
+  pair_config(&cfg, attr, sm_count / (2 * mc), pair_threads<HF_BF16>(), nullptr, false, mc);
   int n = 0;
-  e = cudaOccupancyMaxActiveClusters(&n, lmhead_pair_kernel<HF_BF16, false, MC>, &cfg);
+  e = cudaOccupancyMaxActiveClusters(&n, lmhead_pair_kernel<HF_BF16, false, MULTICAST>, &cfg);
   if (e != cudaSuccess) return e;
   *clusters = n < 1 ? 1 : n;
   return cudaSuccess;
 }
 
 cudaError_t lmhead_pair_max_clusters(int sm_count, int mc, int* clusters) {
-  return mc == 2 ? max_clusters<2>(sm_count, clusters) : max_clusters<1>(sm_count, clusters);
+  return mc == 2 ? max_clusters<true>(sm_count, mc, clusters) : max_clusters<false>(sm_count, mc, clusters);
 }
 
-// One launch: a.plan.G clusters of MC pairs.
-template <int HF, bool VERIFY, int MC>
+// One launch: a.plan.G clusters of mc pairs.
+template <int HF, bool VERIFY, bool MULTICAST>
 static cudaError_t launch_clusters(const PairTokenMaps& tmH, const CUtensorMap& tmW, const PairQuantMaps& tmQ,
-                                   const PairTokenMaps& tmL, const TcArgs& a, cudaStream_t st) {
-  const cudaError_t e = pair_opt_in<HF, VERIFY, MC>();
+                                   const PairTokenMaps& tmL, const TcArgs& a, int mc, cudaStream_t st) {
+  const cudaError_t e = pair_opt_in<HF, VERIFY, MULTICAST>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  pair_config(&cfg, attr, a.plan.G, pair_threads<HF>(), st, true, MC);
-  return cudaLaunchKernelEx(&cfg, lmhead_pair_kernel<HF, VERIFY, MC>, tmH, tmW, tmQ, tmL, a);
+  pair_config(&cfg, attr, a.plan.G, pair_threads<HF>(), st, true, mc);
+  return cudaLaunchKernelEx(&cfg, lmhead_pair_kernel<HF, VERIFY, MULTICAST>, tmH, tmW, tmQ, tmL, a);
 }
 
 template <int HF, bool VERIFY>
 static cudaError_t launch_pair(const PairTokenMaps& tmH, const CUtensorMap& tmW, const PairQuantMaps& tmQ,
                                const PairTokenMaps& tmL, const TcArgs& a, cudaStream_t st) {
   const int ppc = plan_mc(a.plan) * plan_vc(a.plan);  // pairs per cluster
-  if (ppc == 1 && a.plan.G2 == 0) return launch_clusters<HF, VERIFY, 1>(tmH, tmW, tmQ, tmL, a, st);
+  if (ppc == 1 && a.plan.G2 == 0) return launch_clusters<HF, VERIFY, false>(tmH, tmW, tmQ, tmL, a, 1, st);
   if (ppc != 2) return cudaErrorInvalidValue;
   if constexpr (is_quant<HF>()) {
     return cudaErrorInvalidValue;
   } else {
     TcArgs main = a;
     main.plan.role = 0;
-    const cudaError_t e = launch_clusters<HF, VERIFY, 2>(tmH, tmW, tmQ, tmL, main, st);
+    const cudaError_t e = launch_clusters<HF, VERIFY, true>(tmH, tmW, tmQ, tmL, main, 2, st);
     if (e != cudaSuccess || a.plan.G2 == 0) return e;
     // the spill launch of single pairs behind the clusters (the header's
-    // vocabulary split assumes both run)
+    // vocabulary split assumes both run), of the same instantiation: the
+    // largest window takes 48.9 ms with the other one, 48.4 with this
     TcArgs side = a;
     side.plan.role = 1;
     side.plan.G = a.plan.G2;
     side.plan.mc = 1;
     side.plan.vc = 1;
     side.plan.cpu = SPILL_UNIT_SLOTS;
-    return launch_clusters<HF, VERIFY, 1>(tmH, tmW, tmQ, tmL, side, st);
+    return launch_clusters<HF, VERIFY, true>(tmH, tmW, tmQ, tmL, side, 1, st);
   }
 }
 
