@@ -71,7 +71,7 @@ struct BandPlan {
   int G;          // runners that can run at once (CTAs, CTA pairs or clusters)
   int n_vt;       // ceil(V / BN)
   int cpu;        // CTAs per unit: each writes its own partial, so a part has cpu slots
-  int vt_kb;      // KiB of head per v-tile (BN rows as the kernel reads them)
+  int vt_kb;      // KiB of head per v-tile, BN rows as the kernel reads them (no rule reads it)
   int row_bytes;  // bytes of one packed token row as the kernel reads it
   int mc;         // m-tiles a runner holds at once (1, or 2 for 4-CTA clusters sharing head tiles)
   int vc;         // v-tiles a runner takes at once (1, or 2 for 4-CTA clusters sharing token rows)
@@ -114,7 +114,9 @@ __host__ __device__ __forceinline__ int pair_group_rows(int n_rows, int most = 2
 // Rows per group of the SIMT kernel, at most 96, equal sizes rounded up to a
 // multiple of 8 (of 16 above 64). Up to 64 groups, of the four fewest group
 // counts the one whose rounds of tiles times rows cost least, the fewer groups
-// on a tie; the fewest groups beyond.
+// on a tie (LM head, d = 1024, V = 50304: 77 rows as one group of 80 201 us, as
+// two of 40 227; 256 rows as four of 64 625 us, as three of 96 672); the fewest
+// groups beyond.
 __host__ __device__ __forceinline__ int simt_group_rows(const BandPlan& p, int n_rows) {
   if (n_rows <= 0) return 8;
   const int g0 = cdiv(n_rows, 96);

@@ -87,14 +87,10 @@
 //
 // What bounds these heads is the converters' chain of latencies per stage, not
 // the conversion (164 cycles per 64 columns if nothing else ran) nor the MMAs.
-// 294 rows, d = 2048, V = 151936, NVFP4: 123 us, 16 rows 62 us. Decoding into
-// shared memory with one CTA per half v-tile took 208 and 98 us: its chain had
-// the operand stores, a proxy fence and the token rows of a whole group in
-// shared memory besides. With A in tensor memory it went 145 us at 16 rows
-// with a releasing arrive at the peer's barrier (a cluster-scope fence of about
-// 900 cycles each), 80 us with the relaxed one, 75 us with one barrier per
-// 128-column stage, and 62 us with a whole stage per visit of a set instead of
-// 64 columns of it.
+// 294 rows, d = 2048, V = 151936, NVFP4: 121 us, 16 rows 62 us; decoded into
+// shared memory instead, with one CTA per half v-tile, 208 and 98 us (the chain
+// then has the operand stores, a proxy fence and the token rows of a whole
+// group in shared memory besides).
 #include <atomic>
 #include <cstring>
 

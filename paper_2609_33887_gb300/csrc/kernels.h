@@ -93,8 +93,9 @@ cudaError_t launch_lmhead_tc(const CUtensorMap& tmA, const CUtensorMap& tmB, con
                              cudaStream_t st);
 
 // a1+a2 on a CTA pair (tcgen05 cta_group::2), vocabulary on the MMA M side.
-// tmH.m[i] describes hc [P, d] bf16 with 64-column boxes of 16 * (i + 1) rows
-// (one per possible half token group), tmW the head [V, d] bf16 with 64 x 64
+// tmH.m[i] describes hc [P, d] bf16 with 64-column boxes of 8 * (i + 1) rows
+// (half a token group, or the quarter of one that a CTA of two pairs sharing
+// token rows loads), tmW the head [V, d] bf16 with 64 x 64
 // boxes (64 rows: half of a CTA's head rows, see the kernel). plan.G = runners
 // (clusters of plan.mc CTA pairs), plan.BM = 0, plan.cpu = 2.
 struct PairTokenMaps {

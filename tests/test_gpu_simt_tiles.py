@@ -39,8 +39,10 @@ def check_step(h, w, N, V, mid, out, tol):
     assert torch.equal(tok[sure].long(), logit.argmax(1)[sure])
 
 
-# float32 sums of at most 100 products of O(1) numbers (logits of up to ~40) and the base-2 exponential's 2^-22
-TOL = 2e-4
+# float32 sums of at most 100 products with partial sums of up to ~20, whose rounding errors add up like a random walk
+# (four standard deviations: 4 * sqrt(100) * 2^-24 * 20 = 5e-5 on a logit, at most as much on a probability); the
+# base-2 exponential's 2^-22 and the sums over the vocabulary add less than 1e-5
+TOL = 6e-5
 
 
 @pytest.mark.parametrize("N", [1, 7, 8, 9, 33, 40, 63, 64, 65, 77, 129, 200])
