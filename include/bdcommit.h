@@ -239,10 +239,10 @@ int bd_commit_step_ex(const bd_hidden* hidden, const bd_weight* weight,
 size_t bd_workspace_size(const bd_hidden* hidden, const bd_weight* weight,
                          const bd_mask_state* mask_state, const bd_tau_grid* tau_grid);
 
-/* Kernels one bd_commit_step_ex call with these arguments queues (the
- * per-threshold counts' reset is a memset, not a kernel): compaction + row
- * packing, the decode of a quantised head where the LM head reads a bf16
- * copy, the LM head (two launches where spill pairs run beside clusters of
+/* Kernels one bd_commit_step_ex call with these arguments and a workspace of
+ * bd_workspace_size queues: compaction + row packing (and the reset of the
+ * per-threshold counts), the decode of a quantised head where the LM head
+ * reads a bf16 copy, the LM head (two launches where spill pairs run beside clusters of
  * two CTA pairs, see BD_PAIR_SPILL), merge + commit; 0 for an empty window.
  * Arguments as for bd_commit_step_ex (exec may be NULL; only its variant and
  * flags are read). Returns a negative bd_status if the arguments are
