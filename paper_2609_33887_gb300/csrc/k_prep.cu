@@ -213,7 +213,10 @@ __device__ __forceinline__ float pack_row(const __nv_bfloat16* src, int d, uint8
   const int lane = threadIdx.x & 31, nvec = d / 8;
   const uint4* s4 = reinterpret_cast<const uint4*>(src);
   if constexpr (FMT == ROWS_BF16) {
-    constexpr int BATCH = 8;
+    // 12 loads a lane: rows of up to 3072 elements in one batch (223 rows, d =
+    // 2376, V = 35330: 54.9 us a step with 8, 54.3 with 12; with 16, 53.9, but
+    // 4330 rows of d = 4296 lose 0.5%)
+    constexpr int BATCH = 12;
     uint4* d4 = reinterpret_cast<uint4*>(dst);
     for (int v0 = lane; v0 < nvec; v0 += 32 * BATCH) {
       uint4 q[BATCH];
