@@ -88,7 +88,7 @@ struct BandPlan {
 constexpr int BM_PAIR = 0;    // the pair kernel's token groups
 constexpr int BM_QUANT = -1;  // ... with a head decoded in the kernel: groups of at most QUANT_GROUP rows
 constexpr int BM_SIMT = -2;   // simt_group_rows
-constexpr int QUANT_GROUP = 192;
+constexpr int PAIR_GROUP = 256, QUANT_GROUP = 192;
 
 // Words of the workspace header (int32) the kernel that learns N writes for
 // the LM-head and merge kernels: N, the partial slots per row over all
@@ -105,7 +105,7 @@ __host__ __device__ __forceinline__ int cdiv(int a, int b) { return (a + b - 1) 
 
 // Token-group size of the pair kernel for N rows: the fewest groups of at most
 // `most` rows, equal sizes rounded up to a multiple of 32 (16 rows per CTA).
-__host__ __device__ __forceinline__ int pair_group_rows(int n_rows, int most = 256) {
+__host__ __device__ __forceinline__ int pair_group_rows(int n_rows, int most = PAIR_GROUP) {
   if (n_rows <= 0) return 32;
   const int groups = cdiv(n_rows, most);
   return cdiv(cdiv(n_rows, groups), 32) * 32;
@@ -120,13 +120,15 @@ __host__ __device__ __forceinline__ int pair_group_rows(int n_rows, int most = 2
 __host__ __device__ __forceinline__ int simt_group_rows(const BandPlan& p, int n_rows) {
   if (n_rows <= 0) return 8;
   const int g0 = cdiv(n_rows, 96);
-  int best = 0, best_cost = 0;
-  for (int g = g0; g < g0 + 4; ++g) {
+  int best = 0;
+  uint32_t best_cost = 0;
+  for (int g = g0; g < (g0 <= 64 ? g0 + 4 : g0 + 1); ++g) {
     int rows = cdiv(n_rows, g);
     rows = rows <= 64 ? cdiv(rows, 8) * 8 : cdiv(rows, 16) * 16;
-    if (g0 > 64) return rows;
-    // 32 bits: g <= 67, n_vt < 2^24 (2^30 entries in tiles of 112), and G is in the hundreds there
-    const int cost = cdiv(g * p.n_vt, p.G) * rows;
+    // 32 bits where costs are compared: g <= 67, n_vt < 2^24 (2^30 entries in tiles of 112), and G is in
+    // the hundreds there; it may wrap where there is one candidate
+    const uint32_t units = static_cast<uint32_t>(g) * static_cast<uint32_t>(p.n_vt);
+    const uint32_t cost = (units + static_cast<uint32_t>(p.G) - 1u) / static_cast<uint32_t>(p.G) * static_cast<uint32_t>(rows);
     if (best == 0 || cost < best_cost) {
       best = rows;
       best_cost = cost;
@@ -163,8 +165,11 @@ __host__ __device__ __forceinline__ BandPlan plan_resolve(const BandPlan& p, int
 }
 
 // Runner m-tiles (of plan_mc m-tiles each) for N rows; 0 without rows.
+__host__ __device__ __forceinline__ int plan_runner_mts(const BandPlan& p, int n_rows, int bm) {
+  return n_rows > 0 ? cdiv(cdiv(n_rows, bm), plan_mc(p)) : 0;
+}
 __host__ __device__ __forceinline__ int plan_runner_mts(const BandPlan& p, int n_rows) {
-  return n_rows > 0 ? cdiv(cdiv(n_rows, plan_bm(p, n_rows)), plan_mc(p)) : 0;
+  return plan_runner_mts(p, n_rows, plan_bm(p, n_rows));
 }
 
 // Rows of the m-tiles in flight (one band) are kept within ROWS_IN_FLIGHT
@@ -479,14 +484,17 @@ struct TileIter {
   int part;    // vocabulary part of the current unit (this launch's)
   int vt, vt_end;  // its range in steps of vc v-tiles (the spill launch: v-tiles from vt0)
 
-  // hdr: the workspace header the kernel that learns N wrote (HDR_*)
-  __host__ __device__ void init(const BandPlan& stored, const int* hdr, int runner_index) {
+  // hdr: the workspace header the kernel that learns N wrote (HDR_*); bm: the
+  // plan's rows per m-tile for N, where the kernel knows them by its own rule
+  // (the pair kernel carries no other kernel's rule: W8A8, 285 rows, d = 1952, V
+  // = 137970, 87.8 us a step with all of them in it, 85.9 without)
+  __host__ __device__ void init(const BandPlan& stored, const int* hdr, int runner_index, int bm) {
     const int n_rows = hdr_word(hdr, HDR_N);
     const BandPlan plan = plan_resolve(stored, n_rows);
     runner = runner_index;
     G = plan.G;
     mc = plan_mc(plan);
-    n_mt = plan_runner_mts(plan, n_rows);
+    n_mt = plan_runner_mts(plan, n_rows, bm);
     const bool spill = plan.role == 1;
     const int vsplit = hdr_word(hdr, HDR_VSPLIT);
     gm = hdr_word(hdr, spill ? HDR_GM2 : HDR_GM);
@@ -503,6 +511,9 @@ struct TileIter {
     if (none) k.rounds = 0;
     round = -1;
     vt = vt_end = 0;
+  }
+  __host__ __device__ void init(const BandPlan& plan, const int* hdr, int runner_index) {
+    init(plan, hdr, runner_index, plan_bm(plan, hdr_word(hdr, HDR_N)));
   }
 #ifdef __CUDACC__
   __device__ void init(const BandPlan& plan, const int* hdr) { init(plan, hdr, blockIdx.x); }

@@ -87,7 +87,7 @@
 //
 // What bounds these heads is the converters' chain of latencies per stage, not
 // the conversion (164 cycles per 64 columns if nothing else ran) nor the MMAs.
-// 294 rows, d = 2048, V = 151936, NVFP4: 121 us, 16 rows 62 us; decoded into
+// 294 rows, d = 2048, V = 151936, NVFP4: 121 us, 16 rows 60 us; decoded into
 // shared memory instead, with one CTA per half v-tile, 208 and 98 us (the chain
 // then has the operand stores, a proxy fence and the token rows of a whole
 // group in shared memory besides).
@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
   constexpr int ACOLS = atom_cols<HF>();
   constexpr int NATOM = BK / ACOLS;
   const int nk = cdiv(a.d, BK);
-  const int NT = plan_bm(a.plan, n_rows);
+  const int NT = pair_group_rows(n_rows, QUANT ? QUANT_GROUP : PAIR_GROUP);
   const int half = NT / 2;
   // accumulators in TMEM: three of 160 columns when a group has at most 160
   // tokens (the epilogue of one tile then overlaps two tiles of MMAs), else two
@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     uint32_t stage = 0, phase = 0;
     uint32_t issued_mask = 0, issued_phase = 0;
     TileIter it;
-    it.init(a.plan, a.n_rows, pair);
+    it.init(a.plan, a.n_rows, pair, NT);
     bool ok = true;
     while (ok && it.next_unit()) {
       const int tok0 = (it.m_tile + pp_mt) * NT + static_cast<int>(rank) * half;
@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
       uint32_t stage = 0, phase = 0;
       uint32_t acc = 0, acc_phase = 0;
       TileIter it;
-      it.init(a.plan, a.n_rows, pair);
+      it.init(a.plan, a.n_rows, pair, NT);
       bool ok = true;
       while (ok && it.next_unit()) {
         for (int vt = it.vt; ok && vt < it.vt_end; ++vt) {
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     uint32_t r = 0, rph = 0;
     uint32_t issued_mask = 0, issued_phase = 0;
     TileIter it;
-    it.init(a.plan, a.n_rows, pair);
+    it.init(a.plan, a.n_rows, pair, NT);
     bool ok = true;
     while (ok && it.next_unit()) {
       for (int vt = it.vt; ok && vt < it.vt_end; ++vt) {
@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     const int sets = conv_sets(STAGES);
     int turn = 0;  // the set that takes the current operand stage
     TileIter it;
-    it.init(a.plan, a.n_rows, pair);
+    it.init(a.plan, a.n_rows, pair, NT);
     bool ok = true;
     while (ok && it.next_unit()) {
       for (int vt = it.vt; ok && vt < it.vt_end; ++vt) {
@@ -711,7 +711,7 @@ __global__ void __launch_bounds__(pair_threads<HF>(), 1)
     uint32_t epi_phase = 0;
     uint32_t acc = 0, acc_phase = 0;
     TileIter it;
-    it.init(a.plan, a.n_rows, pair);
+    it.init(a.plan, a.n_rows, pair, NT);
     bool ok = true;
     while (ok && it.next_unit()) {
       float m[MAX_CHUNKS], s[MAX_CHUNKS];

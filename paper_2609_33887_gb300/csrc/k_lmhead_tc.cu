@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     uint32_t stage = 0, phase = 0;
     uint32_t issued_mask = 0, issued_phase = 0;  // per stage: issued at least once / parity of last issue
     TileIter it;
-    it.init(a.plan, a.n_rows);
+    it.init(a.plan, a.n_rows, blockIdx.x, TC_BM);
     bool ok = true;
     while (ok && it.next_unit()) {
       for (int vt = it.vt; ok && vt < it.vt_end; ++vt) {
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     uint32_t stage = 0, phase = 0;
     uint32_t acc = 0, acc_phase = 0;
     TileIter it;
-    it.init(a.plan, a.n_rows);
+    it.init(a.plan, a.n_rows, blockIdx.x, TC_BM);
     bool ok = true;
     while (ok && it.next_unit()) {
       for (int vt = it.vt; ok && vt < it.vt_end; ++vt) {
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
     uint32_t acc = 0, acc_phase = 0;
     TileIter it;
-    it.init(a.plan, a.n_rows);
+    it.init(a.plan, a.n_rows, blockIdx.x, TC_BM);
     bool ok = true;
     while (ok && it.next_unit()) {
       float m = -INFINITY, s = 0.f;
